@@ -162,11 +162,11 @@ int debye_ctx::load_plan(const debye_spectra* sp, Plan& pl, cudaStream_t st) {
 
 int debye_ctx::prep_spectra(const debye_spectra* sp, const Plan& pl, cudaStream_t st) {
   int rc;
-  if ((rc = ensure(ws_kf32, sizeof(float4) * 2 * std::max<int64_t>(pl.n_samples, 1), "kf32"))) return rc;
-  if ((rc = ensure(ws_kff, sizeof(float4) * 2 * std::max<int64_t>(pl.n_samples, 1), "kff"))) return rc;
+  if ((rc = ensure(ws_kq, sizeof(float4) * (3 * pl.n_samples + granule_count(pl.n_samples, pl.S)), "sample planes"))) return rc;
   if ((rc = ensure(ws_h0, sizeof(double) * 2 * std::max<int64_t>(pl.S, 1), "h0"))) return rc;
   launch_prep(pl.n_samples, pl.S, sp->offsets, sp->omega, sp->eps_re, sp->eps_im, sp->lo, sp->hi,
-              (float4*)ws_kf32.p, (float4*)ws_kff.p, (double*)ws_h0.p, d_status, sms, st);
+              (float4*)ws_kq.p, (float4*)ws_kq.p + pl.n_samples, (float4*)ws_kq.p + 2 * pl.n_samples,
+              (float4*)ws_kq.p + 3 * pl.n_samples, (double*)ws_h0.p, d_status, sms, st);
   launches += (pl.n_samples > 0) + (pl.S > 0);
   return check_launch("prep");
 }
@@ -225,10 +225,10 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, cudaStream_
   an.units = (const Unit*)ws_tab_units.p;
   an.n_units = (int)gn.units.size();
   an.theta = (const double*)d_th;
-  an.kf32 = (const float4*)ws_kf32.p;
-  an.kff = (const float4*)ws_kff.p;
-  an.kq32 = an.kf32 + pl.n_samples;
-  an.kqff = an.kff + pl.n_samples;
+  an.kq0 = (const float4*)ws_kq.p;
+  an.kq1 = an.kq0 + pl.n_samples;
+  an.kq2 = an.kq1 + pl.n_samples;
+  an.kg = an.kq2 + pl.n_samples;
   an.omega = sp->omega;
   an.eps_re = sp->eps_re;
   an.eps_im = sp->eps_im;
@@ -515,10 +515,10 @@ static int setup_eval(debye_handle h, const debye_spectra* sp, int32_t P, int32_
   if ((rc = h->ensure_scratch(Q, n_max, h->sb_eval, a.sc))) return rc;
   a.units = (const Unit*)h->ws_units.p;
   a.theta = theta;
-  a.kf32 = (const float4*)h->ws_kf32.p;
-  a.kff = (const float4*)h->ws_kff.p;
-  a.kq32 = a.kf32 + pl.n_samples;
-  a.kqff = a.kff + pl.n_samples;
+  a.kq0 = (const float4*)h->ws_kq.p;
+  a.kq1 = a.kq0 + pl.n_samples;
+  a.kq2 = a.kq1 + pl.n_samples;
+  a.kg = a.kq2 + pl.n_samples;
   a.omega = sp->omega;
   a.eps_re = sp->eps_re;
   a.eps_im = sp->eps_im;

@@ -30,11 +30,14 @@ enum Phase { PH_GRAM = 0, PH_REFINE = 1, PH_GRAD = 2, PH_SUMS = 3, PH_SUMSG = 4,
 // Largest pole count with a compile-time (register-resident) column-sum solve;
 // larger ones use the general kernel.
 constexpr int SOLVE_N_MAX = 12;
-// The column sums with the derivative sums (eval.cuh, sums_sq_unit) sweep the
-// samples once for up to this many poles (14 registers per pole) and twice, about
-// N/2 poles each, above it; the cost-only sums (8 registers per pole) always sweep
-// once.
-constexpr int SQUARED_CHUNK_GRAD = 11;
+// The column-sum pass (eval.cuh) sweeps the samples for at most this many poles at a time
+// (8 registers per pole, 14 with the derivative sums), two samples per step: measured on
+// 128 spectra x 512 candidates x 1024 samples at 64 candidates x 2 lanes, N = 12 0.941 ms
+// in sweeps of 6, 1.026 ms with one sample per step, 1.036 ms in one sweep of 12; N = 20
+// 1.558 ms (8 + 6 + 6) against 1.708 ms with one sample per step. Derivative sums, N = 12:
+// 1.723 ms in sweeps of 6, 1.787 ms in sweeps of 4, 1.879 ms with one sample per step.
+constexpr int SQUARED_CHUNK = 8;
+constexpr int SQUARED_CHUNK_GRAD = 6;
 
 struct Unit {
   int32_t s;    // spectrum
@@ -85,14 +88,27 @@ struct TabView {
   const double* lo;        // [S] table origin: the spectrum's lower bound
 };
 
+// Granules of a spectrum: the samples in runs of GRANULE, from its first sample k0; the
+// runs of spectrum s start at granule_base(k0, s) (no two spectra overlap: a spectrum has
+// at most one run more than its samples fill).
+constexpr int GRANULE = 32;
+__host__ __device__ constexpr int64_t granule_base(int64_t k0, int64_t s) { return k0 / GRANULE + s; }
+__host__ __device__ constexpr int64_t granule_count(int64_t n_samples, int64_t S) { return n_samples / GRANULE + S; }
+
 struct EvalArgs {
   const Unit* units;
   int32_t n_units;
   const double* theta;     // [Q][nmax] log10 tau
-  const float4* kf32;      // [sum K] {omega_hi, eps'_hi, eps''_hi, 0}
-  const float4* kff;       // [sum K] {omega_lo, eps'_lo, eps''_lo, 0}
-  const float4* kq32;      // [sum K] {(omega 2^-30)^2, eps', omega eps''} high parts
-  const float4* kqff;      // [sum K] their low parts (float-float)
+  // Samples for the column sums, float-float {high, high, low, low} of one quantity per
+  // plane: kq0 (omega 2^-30)^2, kq1 eps', kq2 omega eps''. Every part is stored twice so
+  // that a 16-byte load gives both operands of the packed FP32 instructions.
+  const float4* kq0;       // [sum K]
+  const float4* kq1;       // [sum K]
+  const float4* kq2;       // [sum K]
+  // Per granule of a spectrum: {smallest (omega 2^-30)^2, largest eps', largest omega eps'',
+  // largest (omega 2^-30)^2}; the second and third are infinite unless every eps' and
+  // omega eps'' of the granule is finite and >= 0.
+  const float4* kg;
   const double* omega;     // [sum K] FP64 inputs
   const double* eps_re;
   const double* eps_im;
@@ -144,24 +160,75 @@ __device__ __forceinline__ void split_double(double v, float& hi, float& lo) {
   lo = __double2float_rn(v - (double)hi);
 }
 
-// acc (hi, lo) += a * b, a and b float-float (one Dot2 step: TwoProduct by FMA,
-// TwoSum of the leading part, low-order terms gathered in lo).
-__device__ __forceinline__ void ff_add_prod(float& ah, float& al, float xh, float xl, float yh,
-                                            float yl) {
-  float p = __fmul_rn(xh, yh);
-  float pe = __fmaf_rn(xh, yh, -p);
-  pe = __fmaf_rn(xh, yl, __fmaf_rn(xl, yh, pe));
-  float s, e;
-  two_sum(ah, p, s, e);
+// ------------------------------------------------------------------ packed FP32
+// The column-sum pass runs its float-float steps on one pole (V = float) or on two poles
+// at once (V = float2, the packed instructions of sm_100 and later: two IEEE operations,
+// rounded as the scalar ones, for one issue slot; measured rate: half the issues of the
+// scalar form at the same FP32 throughput). The v_* operations below are the same for both.
+__device__ __forceinline__ float v_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float v_sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float v_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float v_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float v_neg(float a) { return -a; }
+__device__ __forceinline__ float v_rcp(float a) { return rcp_approx(a); }
+__device__ __forceinline__ float2 v_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 v_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 v_sub(float2 a, float2 b) { return __fadd2_rn(a, v_neg(b)); }
+__device__ __forceinline__ float2 v_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 v_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 v_rcp(float2 a) { return make_float2(rcp_approx(a.x), rcp_approx(a.y)); }
+template <class V> __device__ __forceinline__ V v_all(float a);
+template <> __device__ __forceinline__ float v_all<float>(float a) { return a; }
+template <> __device__ __forceinline__ float2 v_all<float2>(float a) { return make_float2(a, a); }
+// one of a sample's duplicated parts
+__device__ __forceinline__ void v_part(float2 dup, float& v) { v = dup.x; }
+__device__ __forceinline__ void v_part(float2 dup, float2& v) { v = dup; }
+// (max, min) of 1 and a >= 0
+__device__ __forceinline__ void v_order1(float a, float& big, float& small) {
+  big = fmaxf(1.f, a);
+  small = fminf(1.f, a);
+}
+__device__ __forceinline__ void v_order1(float2 a, float2& big, float2& small) {
+  v_order1(a.x, big.x, small.x);
+  v_order1(a.y, big.y, small.y);
+}
+// s + e == a + b exactly: TwoSum, or with ORDERED (the caller knows |a| >= |b|) Dekker's
+// Fast2Sum, whose 3 operations give the same error term.
+template <bool ORDERED, class V>
+__device__ __forceinline__ void v_two_sum(V a, V b, V& s, V& e) {
+  s = v_add(a, b);
+  const V bb = v_sub(s, a);
+  if constexpr (ORDERED) e = v_sub(b, bb);
+  else e = v_add(v_sub(a, v_sub(s, bb)), v_sub(b, bb));
+}
+
+// acc (hi, lo) += a * b, a and b float-float (one Dot2 step: TwoProduct by FMA, exact
+// sum of the leading part, low-order terms gathered in lo).
+template <bool ORDERED, class V>
+__device__ __forceinline__ void v_add_prod(V& ah, V& al, V xh, V xl, V yh, V yl) {
+  const V p = v_mul(xh, yh);
+  V pe = v_fma(xh, yh, v_neg(p));
+  pe = v_fma(xh, yl, v_fma(xl, yh, pe));
+  V s, e;
+  v_two_sum<ORDERED>(ah, p, s, e);
   ah = s;
-  al = __fadd_rn(al, __fadd_rn(e, pe));
+  al = v_add(al, v_add(e, pe));
 }
 
 // Float-float product (ph, pl) = (ah, al) * (bh, bl) to about 2^-46 relative.
-__device__ __forceinline__ void ff_mul(float ah, float al, float bh, float bl, float& ph, float& pl) {
-  ph = __fmul_rn(ah, bh);
-  pl = __fmaf_rn(ah, bh, -ph);
-  pl = __fmaf_rn(ah, bl, __fmaf_rn(al, bh, pl));
+template <class V>
+__device__ __forceinline__ void v_mul_ff(V ah, V al, V bh, V bl, V& ph, V& pl) {
+  ph = v_mul(ah, bh);
+  pl = v_fma(ah, bh, v_neg(ph));
+  pl = v_fma(ah, bl, v_fma(al, bh, pl));
+}
+
+// acc (hi, lo) += x, 0 <= xh <= acc_hi, x float-float (Fast2Sum, exact).
+template <class V>
+__device__ __forceinline__ void v_add_pos(V& ah, V& al, V xh, V xl) {
+  const V s = v_add(ah, xh);
+  al = v_add(al, v_add(v_sub(xh, v_sub(s, ah)), xl));
+  ah = s;
 }
 
 // Float-float value (hi + lo, |lo| <= ulp(hi)/2 after normalisation) for the

@@ -22,6 +22,8 @@
 // No lane returns before the group reduction: lanes without a candidate (the
 // tail of a unit, masked line-search points) contribute zeros.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace debyefit {
@@ -254,23 +256,30 @@ __device__ __forceinline__ void refine_unit(const EvalArgs& a, const Unit& u) {
 }
 
 // ------------------------------------------------------------------ sample staging (bulk copies)
-// The column-sum pass reads, for every sample of a unit's spectrum, the two float4
-// records {(omega 2^-30)^2, eps', omega eps''} (high and low float-float parts);
-// every lane of the block reads the same samples. They are staged in shared memory
-// in chunks of STAGE_SAMPLES by the Tensor Memory Accelerator (cp.async.bulk, a
-// plain global -> shared copy completing on an mbarrier), double-buffered: thread 0
-// issues chunk c + 1 while the block computes on chunk c. Every record is 16 bytes
-// and 16-byte aligned, as the bulk copy requires.
+// The column-sum pass reads, for every sample of a unit's spectrum, one float4 of each
+// of the three sample planes of EvalArgs; every lane of the block reads the same samples.
+// They are staged in shared memory in chunks of STAGE_SAMPLES by the Tensor Memory
+// Accelerator (cp.async.bulk, a plain global -> shared copy completing on an mbarrier),
+// double-buffered: thread 0 issues chunk c + 1 while the block computes on chunk c. Every
+// record is 16 bytes and 16-byte aligned, as the bulk copy requires. The chunk is a
+// multiple of the most lanes per candidate (32), so that a lane's samples keep their
+// stride across chunks; 37 KB per block leave room for 6 blocks per SM. (Chunks of 128,
+// with twice the blocks' room but three times the barriers: 1024 spectra x 8 candidates,
+// 8 lanes each, with the gradient 383 us against 357 us; 256 candidates, one lane each,
+// 1626 against 1597 us.)
 //
 // Every wait on an mbarrier is bounded (STAGE_WAIT_CYCLES of clock64): a wait that
 // runs out records DEBYE_ETIMEOUT, the block agrees on it (__syncthreads_or), waits
 // again, bounded, for its own copies still in flight, and leaves the kernel.
-constexpr int STAGE_SAMPLES = 256;
+constexpr int STAGE_SAMPLES = 384;
+constexpr int STAGE_GRANULES = STAGE_SAMPLES / GRANULE;
+static_assert(STAGE_SAMPLES % GRANULE == 0 && STAGE_SAMPLES % 32 == 0, "a chunk is whole granules and whole lane groups");
+constexpr int STAGE_BUF = 3 * STAGE_SAMPLES + STAGE_GRANULES;   // float4 records of one buffer
+constexpr int STAGE_RECORDS = 2 * STAGE_BUF;
 constexpr long long STAGE_WAIT_CYCLES = 1ll << 31;   // about 1 s at the maximum SM clock
 
 struct Stage {
-  float4* hi;        // [2][STAGE_SAMPLES]
-  float4* lo;        // [2][STAGE_SAMPLES]
+  float4* buf;       // [2][3 planes of STAGE_SAMPLES, then STAGE_GRANULES]
   uint64_t* bar;     // [2] one mbarrier per buffer
   uint32_t fills0, fills1;     // completed phases of each buffer (the same in every thread)
   bool pending0, pending1;     // a copy into the buffer has been issued and not yet waited for
@@ -283,8 +292,7 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
 }
 
 __device__ __forceinline__ void stage_init(Stage& st, float4* buf, uint64_t* bar) {
-  st.hi = buf;
-  st.lo = buf + 2 * STAGE_SAMPLES;
+  st.buf = buf;
   st.bar = bar;
   st.fills0 = st.fills1 = 0;
   st.pending0 = st.pending1 = false;
@@ -296,17 +304,21 @@ __device__ __forceinline__ void stage_init(Stage& st, float4* buf, uint64_t* bar
   __syncthreads();
 }
 
-// Thread 0: copy samples k .. k + n - 1 of both record arrays into buffer b.
-__device__ __forceinline__ void stage_issue(const EvalArgs& a, Stage& st, int b, int64_t k, int n) {
+// Thread 0: copy samples k .. k + n - 1 of the three planes, and their granules (from g),
+// into buffer b.
+__device__ __forceinline__ void stage_issue(const EvalArgs& a, Stage& st, int b, int64_t k, int64_t g, int n) {
   if (threadIdx.x == 0) {
     const uint32_t bytes = (uint32_t)n * (uint32_t)sizeof(float4);
+    const uint32_t gbytes = (uint32_t)((n + GRANULE - 1) / GRANULE) * (uint32_t)sizeof(float4);
     const uint32_t bar = smem_addr(st.bar + b);
+    float4* dst = st.buf + b * STAGE_BUF;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // earlier generic reads of the buffer
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(2u * bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_addr(st.hi + b * STAGE_SAMPLES)), "l"(a.kq32 + k), "r"(bytes), "r"(bar) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_addr(st.lo + b * STAGE_SAMPLES)), "l"(a.kqff + k), "r"(bytes), "r"(bar) : "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(3u * bytes + gbytes) : "memory");
+    const float4* src[4] = {a.kq0 + k, a.kq1 + k, a.kq2 + k, a.kg + g};
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   ::"r"(smem_addr(dst + p * STAGE_SAMPLES)), "l"(src[p]), "r"(p < 3 ? bytes : gbytes), "r"(bar) : "memory");
   }
   st.pending(b) = true;
 }
@@ -355,7 +367,7 @@ __device__ __forceinline__ bool stage_wait(const EvalArgs& a, Stage& st, int b) 
 // With im = x re = omega tau re,
 //   h_i = sum_k re_i(k) eps'_k + tau_i B_i,   B_i = sum_k re_i(k) (omega_k eps''_k),
 // two Dot2 sums on the per-sample eps' and omega eps'' (k_prep_samples stores
-// {omega^2, eps', omega eps''} in a.kq32 / a.kqff). With u = x^2 re^2 = re (1 - re),
+// omega^2, eps' and omega eps'' in a.kq0, a.kq1, a.kq2). With u = x^2 re^2 = re (1 - re),
 // d re / d theta = -2 ln10 u and d im / d theta = ln10 x re^2 (1 - x^2)
 // = ln10 omega tau (re - 2u), so
 //   D_i = -2 ln10 U_i,   E_i = ln10 (-2 V_i + tau_i (B_i - 2 W_i)),
@@ -366,140 +378,276 @@ __device__ __forceinline__ bool stage_wait(const EvalArgs& a, Stage& st, int b) 
 // in the solve), sc.G[i Q + q] = S_i, sc.G[(N + i) Q + q] = h_i, and with GRAD
 // sc.G[(2N + i) Q + q] = D_i, sc.G[(3N + i) Q + q] = E_i.
 //
-// One sweep over the samples for poles P0 .. P0 + C - 1 of an N-pole candidate:
+// The steps of one pole (V = float) or of a pair of poles (V = float2).
+template <class V, bool GRAD>
+struct SumAcc {
+  V t2h, t2l;                       // (tau 2^30)^2
+  V sh, sl, ah, al, ch, cl;         // S + 1, sum re eps', sum re omega eps''
+  V uh, ul, vh, vl, wh, wl;         // GRAD: U + 1, V, W
+};
+
+// One sample of the three planes, every part twice.
+struct SamplePair {
+  float2 w2h, w2l, erh, erl, cih, cil;
+  __device__ __forceinline__ void load(const float4* p) {
+    const float4 a = p[0], b = p[STAGE_SAMPLES], c = p[2 * STAGE_SAMPLES];
+    w2h = make_float2(a.x, a.y);
+    w2l = make_float2(a.z, a.w);
+    erh = make_float2(b.x, b.y);
+    erl = make_float2(b.z, b.w);
+    cih = make_float2(c.x, c.y);
+    cil = make_float2(c.z, c.w);
+  }
+};
+
+template <bool ORDERED, class V, bool GRAD>
+__device__ __forceinline__ void sums_sq_step(SumAcc<V, GRAD>& t, const SamplePair& smp) {
+  V w2h, w2l, erh, erl, cih, cil;
+  v_part(smp.w2h, w2h);
+  v_part(smp.w2l, w2l);
+  v_part(smp.erh, erh);
+  v_part(smp.erl, erl);
+  v_part(smp.cih, cih);
+  v_part(smp.cil, cil);
+  // x^2 in float-float (the product of the low parts, ~2^-48, is dropped)
+  const V x2h = v_mul(w2h, t.t2h);
+  V x2l = v_fma(w2h, t.t2h, v_neg(x2h));
+  x2l = v_fma(w2h, t.t2l, v_fma(w2l, t.t2h, x2l));
+  // d = 1 + x^2: Fast2Sum of (max, min), exact
+  V big, small;
+  v_order1(x2h, big, small);
+  const V dh = v_add(big, small);
+  const V dl = v_add(v_sub(small, v_sub(dh, big)), x2l);
+  // re = 1/d: approximate reciprocal and one Newton step on the float-float d
+  const V r0 = v_rcp(dh);
+  V e = v_fma(v_neg(dh), r0, v_all<V>(1.0f));
+  e = v_fma(v_neg(dl), r0, e);
+  const V rl = v_mul(r0, e);
+  v_add_pos(t.sh, t.sl, r0, rl);                         // sh >= 1 >= re
+  v_add_prod<ORDERED>(t.ah, t.al, r0, rl, erh, erl);              // re eps'
+  v_add_prod<ORDERED>(t.ch, t.cl, r0, rl, cih, cil);              // re omega eps''
+  if constexpr (GRAD) {
+    V r2h, r2l, qh, ql;
+    v_mul_ff(r0, rl, r0, rl, r2h, r2l);                  // re^2
+    v_mul_ff(x2h, x2l, r2h, r2l, qh, ql);                // u = x^2 re^2
+    v_add_pos(t.uh, t.ul, qh, ql);                       // uh >= 1 >= u
+    v_add_prod<ORDERED>(t.vh, t.vl, qh, ql, erh, erl);            // u eps'
+    v_add_prod<ORDERED>(t.wh, t.wl, qh, ql, cih, cil);            // u omega eps''
+  }
+}
+
+__device__ __forceinline__ float& v_half(float2& v, int k) { return k ? v.y : v.x; }
+__device__ __forceinline__ float& v_half(float& v, int) { return v; }
+
+// tau = 10^theta of pole j and the float-float (tau 2^30)^2. One call site per kernel
+// serves every pole: the FP64 power is about 25 FP64 instructions, each of which holds a
+// sub-partition's FP64 pipe for 64 cycles on this GPU.
+static __device__ __noinline__ double sums_tau(double theta, float& h, float& l) {
+  const double tau = exp10(theta);
+  const double ts = tau * 0x1p30;
+  split_double(ts * ts, h, l);
+  return tau;
+}
+
+template <class V, bool GRAD>
+__device__ __forceinline__ void sums_sq_zero(SumAcc<V, GRAD>& t, int k) {
+  v_half(t.sh, k) = 1.f;
+  v_half(t.sl, k) = v_half(t.ah, k) = v_half(t.al, k) = v_half(t.ch, k) = v_half(t.cl, k) = 0.f;
+  if constexpr (GRAD) {
+    v_half(t.uh, k) = 1.f;
+    v_half(t.ul, k) = v_half(t.vh, k) = v_half(t.vl, k) = v_half(t.wh, k) = v_half(t.wl, k) = 0.f;
+  }
+}
+
+// The group's totals of one pole.
+template <bool GRAD>
+struct PoleSums {
+  float sh, sl, ah, al, ch, cl, uh, ul, vh, vl, wh, wl;
+  template <class V>
+  __device__ __forceinline__ void reduce(SumAcc<V, GRAD>& t, int k, int ks) {
+    sh = v_half(t.sh, k), sl = v_half(t.sl, k), ah = v_half(t.ah, k), al = v_half(t.al, k);
+    ch = v_half(t.ch, k), cl = v_half(t.cl, k);
+    group_sum_ff(sh, sl, ks);
+    group_sum_ff(ah, al, ks);
+    group_sum_ff(ch, cl, ks);
+    if constexpr (GRAD) {
+      uh = v_half(t.uh, k), ul = v_half(t.ul, k), vh = v_half(t.vh, k), vl = v_half(t.vl, k);
+      wh = v_half(t.wh, k), wl = v_half(t.wl, k);
+      group_sum_ff(uh, ul, ks);
+      group_sum_ff(vh, vl, ks);
+      group_sum_ff(wh, wl, ks);
+    }
+  }
+  // S, h (and D, E) of pole j of candidate q in FP64
+  template <int N>
+  __device__ __forceinline__ void write(const EvalArgs& a, int q, int j, int ks) const {
+    double* G = a.sc.G;
+    const int64_t Q = a.sc.Q;
+    constexpr double LN10 = 2.302585092994046;
+    const double tau = a.sc.x[(int64_t)j * Q + q];
+    const double B = (double)ch + (double)cl;
+    G[(int64_t)j * Q + q] = ((double)sh - (double)ks) + (double)sl;
+    G[(int64_t)(N + j) * Q + q] = ((double)ah + (double)al) + tau * B;
+    if constexpr (GRAD) {
+      const double U = ((double)uh - (double)ks) + (double)ul;
+      const double Vs = (double)vh + (double)vl;
+      const double W = (double)wh + (double)wl;
+      G[(int64_t)(2 * N + j) * Q + q] = -2.0 * LN10 * U;
+      G[(int64_t)(3 * N + j) * Q + q] = LN10 * (-2.0 * Vs + tau * (B - 2.0 * W));
+    }
+  }
+};
+
+// Every product that a granule adds to the sums of half k of t is at most the accumulator
+// it is added to: re <= 1 / (1 + w2min tau^2) and u = re (1 - re) <= min(re, 1/4, x^2) up
+// to rounding (2^-21, covered by the factor), and the accumulators only grow while the
+// granule's values are >= 0. The granule's infinite bounds compare false.
+template <class V, bool GRAD>
+__device__ __forceinline__ bool sums_sq_ordered(SumAcc<V, GRAD>& t, int k, float4 g) {
+  const float t2 = v_half(t.t2h, k);
+  const float re = rcp_approx(__fmaf_rn(g.x, t2, 1.f)) * 1.00001f;
+  bool ok = v_half(t.ah, k) >= g.y * re && v_half(t.ch, k) >= g.z * re;
+  if constexpr (GRAD) {
+    const float u = fminf(fminf(re, 0.25f), g.w * t2) * 1.00001f;
+    ok = ok && v_half(t.vh, k) >= g.y * u && v_half(t.wh, k) >= g.z * u;
+  }
+  return ok;
+}
+
+// One sweep over the samples for poles P0 .. P0 + C - 1 of an N-pole candidate, two poles
+// per packed step (an odd last pole takes the scalar step). The FP64 work per pole (tau,
+// and the final sums) is dealt out to the group's lanes, pole i to lane i mod ks.
+//
+// What bounds it: operand reads from the register file. A packed addition reads 4
+// registers and a packed FMA 6 of the 2 that a sub-partition delivers per cycle (measured
+// 2.0 and 3.0 cycles per warp instruction), so the 40 operations of a (sample, pole)
+// cannot run at the FP32 pipe's 40 cycles; scalar instructions cost the same reads at
+// twice the issue slots (62 cycles per (sample, pole) for N = 12 before, 57 packed). What
+// is left is to issue fewer of them: where a granule's bounds show that no product can
+// exceed the accumulator it is added to, the exact sum needs 3 additions instead of 6,
+// with the same error term. 47 cycles now: N = 12, 128 spectra x 512 candidates x 1024
+// samples at 64 candidates x 2 lanes 1.259 -> 0.941 ms, N = 20 2.512 -> 1.558 ms, N = 2
+// 0.233 -> 0.184 ms; derivative sums N = 8 1.474 -> 1.158 ms. Every rounding is unchanged.
 template <int N, int P0, int C, bool GRAD>
 __device__ __forceinline__ bool sums_sq_sweep(const EvalArgs& a, const Unit& u, const Lane& ln, int q, Stage& st) {
-  const double* th = a.theta + (int64_t)q * a.sc.nmax + P0;
-  const int64_t Q = a.sc.Q;
-  constexpr int CG = GRAD ? C : 1;
-  float t2h[C], t2l[C], sh[C], sl[C], ah[C], al[C], ch[C], cl[C];
-  float uh[CG], ul[CG], vh_[CG], vl_[CG], wh[CG], wl[CG];
+  constexpr int CP = C / 2, ODD = C & 1;
+  constexpr unsigned FULL = 0xffffffffu;
+  SumAcc<float2, GRAD> pr[CP > 0 ? CP : 1];
+  SumAcc<float, GRAD> odd;
+  float mh = 0.f, ml = 0.f;
 #pragma unroll
   for (int i = 0; i < C; ++i) {
-    t2h[i] = t2l[i] = 0.f;
-    if (ln.act) {
-      const double t = exp10(th[i]);
-      const double ts = t * 0x1p30;
-      split_double(ts * ts, t2h[i], t2l[i]);
-      if (ln.slice == 0) a.sc.x[(int64_t)(P0 + i) * Q + q] = t;   // tau for k_solve_sums and the epilogue
+    const int own = i & (ln.ks - 1);
+    if (own == 0) {
+      const int j = P0 + i + ln.slice;
+      mh = ml = 0.f;
+      if (ln.act && i + ln.slice < C) a.sc.x[(int64_t)j * a.sc.Q + q] = sums_tau(a.theta[(int64_t)q * a.sc.nmax + j], mh, ml);
     }
-    sh[i] = 1.f;
-    sl[i] = ah[i] = al[i] = ch[i] = cl[i] = 0.f;
+    const float h = __shfl_sync(FULL, mh, own, ln.ks), l = __shfl_sync(FULL, ml, own, ln.ks);
+    if (i < 2 * CP) {
+      v_half(pr[i / 2].t2h, i & 1) = h;
+      v_half(pr[i / 2].t2l, i & 1) = l;
+      sums_sq_zero(pr[i / 2], i & 1);
+    } else {
+      odd.t2h = h;
+      odd.t2l = l;
+      sums_sq_zero(odd, 0);
+    }
   }
-#pragma unroll
-  for (int i = 0; i < CG; ++i) {
-    uh[i] = 1.f;
-    ul[i] = vh_[i] = vl_[i] = wh[i] = wl[i] = 0.f;
-  }
-  const int64_t nk = u.k1 - u.k0;
+  const int64_t nk = u.k1 - u.k0, g0 = granule_base(u.k0, u.s);
   const int nch = (int)((nk + STAGE_SAMPLES - 1) / STAGE_SAMPLES);
   auto chunk_len = [&](int64_t c0) { return (int)(nk - c0 < STAGE_SAMPLES ? nk - c0 : STAGE_SAMPLES); };
-  if (nch > 0) stage_issue(a, st, 0, u.k0, chunk_len(0));
+  // Samples per check of the order: 16 of every lane; from 8 lanes on the whole chunk (a
+  // check per 128 samples costs more than the ordered sums gain there: 1024 spectra x 8
+  // candidates with the gradient 369 us against 357 us)
+  const int run = ln.ks <= 2 ? GRANULE : ln.ks <= 4 ? 2 * GRANULE : STAGE_SAMPLES;
+  if (nch > 0) stage_issue(a, st, 0, u.k0, g0, chunk_len(0));
 #pragma unroll 1
   for (int c = 0; c < nch; ++c) {
     const int b = c & 1;
     const int64_t c0 = (int64_t)c * STAGE_SAMPLES;
     if (c + 1 < nch)   // buffer b ^ 1 was released by the barrier that ended chunk c - 1
-      stage_issue(a, st, b ^ 1, u.k0 + c0 + STAGE_SAMPLES, chunk_len(c0 + STAGE_SAMPLES));
+      stage_issue(a, st, b ^ 1, u.k0 + c0 + STAGE_SAMPLES, g0 + (int64_t)(c + 1) * STAGE_GRANULES,
+                  chunk_len(c0 + STAGE_SAMPLES));
     if (!stage_wait(a, st, b)) return false;
+    const float4* buf = st.buf + b * STAGE_BUF;
     const int cnt = chunk_len(c0);
-    const float4* bh = st.hi + b * STAGE_SAMPLES;
-    const float4* bl = st.lo + b * STAGE_SAMPLES;
-    const int jend = ln.act ? cnt : 0;
-    float4 vhn = bh[ln.slice < jend ? ln.slice : 0], vln = bl[ln.slice < jend ? ln.slice : 0];
 #pragma unroll 1
-  for (int j = ln.slice; j < jend; j += ln.ks) {
-    const float4 vh = vhn, vl = vln;
-    if (j + ln.ks < jend) {   // next sample's records in flight during this one
-      vhn = bh[j + ln.ks];
-      vln = bl[j + ln.ks];
-    }
-#pragma unroll
-    for (int i = 0; i < C; ++i) {
-      // x^2 in float-float (the product of the low parts, ~2^-48, is dropped)
-      const float x2h = __fmul_rn(vh.x, t2h[i]);
-      float x2l = __fmaf_rn(vh.x, t2h[i], -x2h);
-      x2l = __fmaf_rn(vh.x, t2l[i], __fmaf_rn(vl.x, t2h[i], x2l));
-      // d = 1 + x^2: Fast2Sum of (max, min), exact
-      const float big = fmaxf(1.f, x2h), small = fminf(1.f, x2h);
-      const float dh = __fadd_rn(big, small);
-      const float dl = __fadd_rn(__fsub_rn(small, __fsub_rn(dh, big)), x2l);
-      // re = 1/d: approximate reciprocal and one Newton step on the float-float d
-      const float r0 = rcp_approx(dh);
-      float e = __fmaf_rn(-dh, r0, 1.0f);
-      e = __fmaf_rn(-dl, r0, e);
-      const float rl = __fmul_rn(r0, e);
-      const float gs = __fadd_rn(sh[i], r0);                         // Fast2Sum, sh >= 1 >= re
-      sl[i] = __fadd_rn(sl[i], __fadd_rn(__fsub_rn(r0, __fsub_rn(gs, sh[i])), rl));
-      sh[i] = gs;
-      ff_add_prod(ah[i], al[i], r0, rl, vh.y, vl.y);                 // re eps'
-      ff_add_prod(ch[i], cl[i], r0, rl, vh.z, vl.z);                 // re omega eps''
-      if constexpr (GRAD) {
-        float r2h, r2l, qh, ql;
-        ff_mul(r0, rl, r0, rl, r2h, r2l);                            // re^2
-        ff_mul(x2h, x2l, r2h, r2l, qh, ql);                          // u = x^2 re^2
-        const float gu = __fadd_rn(uh[i], qh);                       // Fast2Sum, uh >= 1 >= u
-        ul[i] = __fadd_rn(ul[i], __fadd_rn(__fsub_rn(qh, __fsub_rn(gu, uh[i])), ql));
-        uh[i] = gu;
-        ff_add_prod(vh_[i], vl_[i], qh, ql, vh.y, vl.y);             // u eps'
-        ff_add_prod(wh[i], wl[i], qh, ql, vh.z, vl.z);               // u omega eps''
+    for (int jb = 0; jb < cnt; jb += run) {
+      const int je = jb + run < cnt ? jb + run : cnt;
+      float4 g = buf[3 * STAGE_SAMPLES + jb / GRANULE];
+      for (int gi = jb + GRANULE; gi < je; gi += GRANULE) {
+        const float4 h = buf[3 * STAGE_SAMPLES + gi / GRANULE];
+        g = make_float4(fminf(g.x, h.x), fmaxf(g.y, h.y), fmaxf(g.z, h.z), fmaxf(g.w, h.w));
       }
+      bool fast = true;
+#pragma unroll
+      for (int i = 0; i < CP; ++i) fast = fast && sums_sq_ordered(pr[i], 0, g) && sums_sq_ordered(pr[i], 1, g);
+      if constexpr (ODD) fast = fast && sums_sq_ordered(odd, 0, g);
+      const int jend = ln.act ? je : 0;
+      auto sweep = [&](auto ordered) {
+        constexpr bool ORD = decltype(ordered)::value;
+        constexpr int U = 2;   // samples per step: their reciprocals and products overlap
+        int j = jb + ln.slice;
+        auto one = [&](const SamplePair& smp) {
+#pragma unroll
+          for (int i = 0; i < CP; ++i) sums_sq_step<ORD>(pr[i], smp);
+          if constexpr (ODD) sums_sq_step<ORD>(odd, smp);
+        };
+#pragma unroll 1
+        for (; j + (U - 1) * ln.ks < jend; j += U * ln.ks) {
+          SamplePair smp[U];
+#pragma unroll
+          for (int v = 0; v < U; ++v) smp[v].load(buf + j + v * ln.ks);
+#pragma unroll
+          for (int v = 0; v < U; ++v) one(smp[v]);
+        }
+#pragma unroll 1
+        for (; j < jend; j += ln.ks) {
+          SamplePair smp;
+          smp.load(buf + j);
+          one(smp);
+        }
+      };
+      if (__all_sync(FULL, fast || !ln.act)) sweep(std::true_type{});
+      else sweep(std::false_type{});
     }
-  }
     __syncthreads();   // the whole block is done with buffer b
   }
+  PoleSums<GRAD> mine, t;
 #pragma unroll
   for (int i = 0; i < C; ++i) {
-    group_sum_ff(sh[i], sl[i], ln.ks);
-    group_sum_ff(ah[i], al[i], ln.ks);
-    group_sum_ff(ch[i], cl[i], ln.ks);
-  }
-#pragma unroll
-  for (int i = 0; i < CG; ++i) {
-    if constexpr (GRAD) {
-      group_sum_ff(uh[i], ul[i], ln.ks);
-      group_sum_ff(vh_[i], vl_[i], ln.ks);
-      group_sum_ff(wh[i], wl[i], ln.ks);
-    }
-  }
-  if (ln.act && ln.slice == 0) {
-    double* G = a.sc.G;
-    constexpr double LN10 = 2.302585092994046;
-#pragma unroll
-    for (int i = 0; i < C; ++i) {
-      const int64_t j = P0 + i;
-      const double t = a.sc.x[j * Q + q];
-      const double B = (double)ch[i] + (double)cl[i];
-      G[j * Q + q] = ((double)sh[i] - (double)ln.ks) + (double)sl[i];
-      G[(N + j) * Q + q] = ((double)ah[i] + (double)al[i]) + t * B;
-      if constexpr (GRAD) {
-        const double U = ((double)uh[i] - (double)ln.ks) + (double)ul[i];
-        const double V = (double)vh_[i] + (double)vl_[i];
-        const double W = (double)wh[i] + (double)wl[i];
-        G[(2 * N + j) * Q + q] = -2.0 * LN10 * U;
-        G[(3 * N + j) * Q + q] = LN10 * (-2.0 * V + t * (B - 2.0 * W));
-      }
+    const int own = i & (ln.ks - 1);
+    if (i < 2 * CP) t.reduce(pr[i / 2], i & 1, ln.ks);
+    else t.reduce(odd, 0, ln.ks);
+    if (own == ln.slice) mine = t;
+    if (own == ln.ks - 1 || i == C - 1) {
+      const int k = i - own + ln.slice;   // this lane's pole of the group's last ks poles
+      if (ln.act && k < C) mine.template write<N>(a, q, P0 + k, ln.ks);
     }
   }
   return true;
 }
 
-// With GRAD, more than SQUARED_CHUNK_GRAD poles take two sweeps of about N/2 poles
-// each (14 registers per pole); the cost-only sums (8 per pole) sweep once. A unit
-// without any active candidate (a masked evaluation) is skipped by the whole block.
+// Poles P0 .. N - 1 in sweeps of at most CH poles each, an even number wherever possible.
+template <int N, int P0, int CH, bool GRAD>
+__device__ __forceinline__ bool sums_sq_sweeps(const EvalArgs& a, const Unit& u, const Lane& ln, int q, Stage& st) {
+  constexpr int REST = N - P0, NS = (REST + CH - 1) / CH;          // sweeps still to make
+  constexpr int EVEN = ((REST + NS - 1) / NS + 1) / 2 * 2;         // their size, rounded up to even
+  constexpr int C = EVEN < REST ? (EVEN <= CH ? EVEN : CH) : REST;
+  if (!sums_sq_sweep<N, P0, C, GRAD>(a, u, ln, q, st)) return false;
+  if constexpr (P0 + C < N) return sums_sq_sweeps<N, P0 + C, CH, GRAD>(a, u, ln, q, st);
+  return true;
+}
+
+// A unit without any active candidate (a masked evaluation) is skipped by the whole block.
 // Returns false if a wait for staged samples ran out (the block then stops).
 template <int N, bool GRAD>
 __device__ __forceinline__ bool sums_sq_unit(const EvalArgs& a, const Unit& u, Stage& st) {
   const Lane ln = lane_of(a, u, false);
   if (!__syncthreads_or(ln.act)) return true;
   const int q = ln.act ? ln.q : u.q0;
-  if constexpr (!GRAD || N <= SQUARED_CHUNK_GRAD) {
-    return sums_sq_sweep<N, 0, N, GRAD>(a, u, ln, q, st);
-  } else {
-    constexpr int C1 = (N + 1) / 2;
-    if (!sums_sq_sweep<N, 0, C1, GRAD>(a, u, ln, q, st)) return false;
-    return sums_sq_sweep<N, C1, N - C1, GRAD>(a, u, ln, q, st);
-  }
+  return sums_sq_sweeps<N, 0, GRAD ? SQUARED_CHUNK_GRAD : SQUARED_CHUNK, GRAD>(a, u, ln, q, st);
 }
 
 // ------------------------------------------------------------------ gradient pass
@@ -611,7 +759,7 @@ __device__ __forceinline__ void dispatch_n(const EvalArgs& a, const Unit& u) {
 // (grid-stride over the unit list), the unit's samples staged by bulk copies.
 template <int N, bool GRAD, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) k_pass_sums(EvalArgs a) {
-  __shared__ __align__(128) float4 stage_buf[4 * STAGE_SAMPLES];
+  __shared__ __align__(128) float4 stage_buf[STAGE_RECORDS];
   __shared__ __align__(8) uint64_t stage_bar[2];
   Stage st;
   stage_init(st, stage_buf, stage_bar);

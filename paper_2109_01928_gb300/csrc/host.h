@@ -68,7 +68,7 @@ struct debye_ctx {
   cudaStream_t side[debyefit::N_BUCKETS] = {nullptr};
   cudaEvent_t ev_fork = nullptr, ev_join[debyefit::N_BUCKETS] = {nullptr};
 
-  debyefit::Buf ws_kf32, ws_kff, ws_h0, ws_units;
+  debyefit::Buf ws_kq, ws_h0, ws_units;
   debyefit::Buf ws_tab_units;    // units of the column-sum tables' node pass
   debyefit::TabView tab{};       // column-sum tables of the current call (DEBYE_PREC_MIXED_TABLE)
   debyefit::ScratchBufs sb_eval, sb_polish, sb_polish_acc, sb_final;
@@ -118,8 +118,7 @@ struct debye_ctx {
     b.n = 0;
   }
   void release() {
-    free_buf(ws_kf32);
-    free_buf(ws_kff);
+    free_buf(ws_kq);
     free_buf(ws_h0);
     free_buf(ws_units);
     free_buf(ws_tab_units);

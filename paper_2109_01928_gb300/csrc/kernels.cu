@@ -10,42 +10,59 @@
 namespace debyefit {
 
 // ------------------------------------------------------------------ input preparation
-// Per sample: float-float split of omega, eps', eps'' for the mixed passes (the
-// first n records of kf32 / kff) and of (omega 2^-30)^2, eps', omega eps'' for the
-// squared-form column sums (records n .. 2n - 1), and finiteness checks; per
-// spectrum: h0 = sum_k eps'_k and b^T b (FP64).
+// Per sample: float-float splits of (omega 2^-30)^2, eps' and omega eps'' for the column
+// sums (the planes of EvalArgs), and finiteness checks; per spectrum: h0 = sum_k eps'_k
+// and b^T b (FP64).
 __global__ void k_prep_samples(int64_t n, const double* __restrict__ omega,
                                const double* __restrict__ er, const double* __restrict__ ei,
-                               float4* __restrict__ kf32, float4* __restrict__ kff, int* status) {
+                               float4* __restrict__ kq0, float4* __restrict__ kq1, float4* __restrict__ kq2,
+                               int* status) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
     const double w = omega[k], a = er[k], b = ei[k];
     if (!(w > 0.0) || !isfinite(w) || !isfinite(a) || !isfinite(b)) set_status(status, DEBYE_ENOTFINITE);
-    float wh, wl, ah, al, bh, bl, w2h, w2l, ch, cl;
-    split_double(w, wh, wl);
-    split_double(a, ah, al);
-    split_double(b, bh, bl);
-    kf32[k] = make_float4(wh, ah, bh, 0.f);
-    kff[k] = make_float4(wl, al, bl, 0.f);
+    float h, l;
     const double ws = w * 0x1p-30;
-    split_double(ws * ws, w2h, w2l);
-    split_double(w * b, ch, cl);
-    kf32[n + k] = make_float4(w2h, ah, ch, 0.f);
-    kff[n + k] = make_float4(w2l, al, cl, 0.f);
+    split_double(ws * ws, h, l);
+    kq0[k] = make_float4(h, h, l, l);
+    split_double(a, h, l);
+    kq1[k] = make_float4(h, h, l, l);
+    split_double(w * b, h, l);
+    kq2[k] = make_float4(h, h, l, l);
   }
 }
 
-__global__ void k_prep_spectra(int64_t S, const int64_t* __restrict__ offsets,
+// One block per spectrum; each warp's 32 samples of an iteration are one granule.
+__global__ void k_prep_spectra(int64_t S, const int64_t* __restrict__ offsets, const double* __restrict__ omega,
                                const double* __restrict__ er, const double* __restrict__ ei,
                                const double* __restrict__ lo, const double* __restrict__ hi,
-                               double* __restrict__ h0, double* __restrict__ bb, int* status) {
+                               double* __restrict__ h0, double* __restrict__ bb, float4* __restrict__ kg,
+                               int* status) {
+  static_assert(GRANULE == 32, "a granule is a warp's samples");
   __shared__ double red[32], red2[32];
   for (int64_t s = blockIdx.x; s < S; s += gridDim.x) {
     const int64_t a = offsets[s], b = offsets[s + 1];
     double acc = 0.0, acc2 = 0.0;
-    for (int64_t k = a + threadIdx.x; k < b; k += blockDim.x) {
-      acc += er[k];
-      acc2 = fma(er[k], er[k], fma(ei[k], ei[k], acc2));
+    for (int64_t k0 = a + (threadIdx.x & ~31u); k0 < b; k0 += blockDim.x) {
+      const int64_t k = k0 + (threadIdx.x & 31);
+      float w2lo = INFINITY, w2hi = 0.f, e = 0.f, c = 0.f;   // neutral for the lanes past the spectrum's end
+      if (k < b) {
+        const double w = omega[k], r = er[k], i = ei[k], ws = w * 0x1p-30;
+        acc += r;
+        acc2 = fma(r, r, fma(i, i, acc2));
+        w2lo = __double2float_rd(ws * ws);
+        w2hi = __double2float_ru(ws * ws);
+        e = __double2float_rn(r);
+        c = __double2float_rn(w * i);
+        if (!(e >= 0.f && e < INFINITY && c >= 0.f && c < INFINITY && w2lo >= 0.f)) e = c = INFINITY;
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        w2lo = fminf(w2lo, __shfl_xor_sync(0xffffffffu, w2lo, o));
+        w2hi = fmaxf(w2hi, __shfl_xor_sync(0xffffffffu, w2hi, o));
+        e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
+        c = fmaxf(c, __shfl_xor_sync(0xffffffffu, c, o));
+      }
+      if ((threadIdx.x & 31) == 0) kg[granule_base(a, s) + (k0 - a) / GRANULE] = make_float4(w2lo, e, c, w2hi);
     }
     for (int o = 16; o > 0; o >>= 1) {
       acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -563,14 +580,15 @@ __global__ void __launch_bounds__(256) k_grad_finish(EvalArgs a, double* grad) {
 // ------------------------------------------------------------------ host launchers
 void launch_prep(int64_t n_samples, int64_t S, const int64_t* offsets, const double* omega,
                  const double* er, const double* ei, const double* lo, const double* hi,
-                 float4* kf32, float4* kff, double* h0, int* status, int sms, cudaStream_t st) {
+                 float4* kq0, float4* kq1, float4* kq2, float4* kg, double* h0, int* status, int sms,
+                 cudaStream_t st) {
   if (n_samples > 0) {
     int grid = (int)std::min<int64_t>((n_samples + 255) / 256, (int64_t)sms * 16);
-    k_prep_samples<<<grid, 256, 0, st>>>(n_samples, omega, er, ei, kf32, kff, status);
+    k_prep_samples<<<grid, 256, 0, st>>>(n_samples, omega, er, ei, kq0, kq1, kq2, status);
   }
   if (S > 0) {
     int grid = (int)std::min<int64_t>(S, (int64_t)sms * 8);
-    k_prep_spectra<<<grid, 256, 0, st>>>(S, offsets, er, ei, lo, hi, h0, h0 + S, status);
+    k_prep_spectra<<<grid, 256, 0, st>>>(S, offsets, omega, er, ei, lo, hi, h0, h0 + S, kg, status);
   }
 }
 

@@ -66,11 +66,12 @@ inline void launch_pass(int N, int phase, const EvalArgs& a, int grid, int block
   }
 }
 
-// kf32, kff: [2 n_samples] records (the second half for the squared-form column sums);
+// kq0, kq1, kq2: [n_samples] each, the sample planes of EvalArgs; kg: [granule_count];
 // h0: [2 S] doubles, sum_k eps'_k per spectrum, then b^T b per spectrum.
 void launch_prep(int64_t n_samples, int64_t S, const int64_t* offsets, const double* omega,
                  const double* er, const double* ei, const double* lo, const double* hi,
-                 float4* kf32, float4* kff, double* h0, int* status, int sms, cudaStream_t st);
+                 float4* kq0, float4* kq1, float4* kq2, float4* kg, double* h0, int* status, int sms,
+                 cudaStream_t st);
 // Mixed evaluation after the column-sum pass: weights, flip, cost and (grad != nullptr,
 // after the pass with derivative sums) the gradient in theta.
 void launch_solve_sums(const EvalArgs& a, double* cost, double* weights, double* grad, int block, int sms,

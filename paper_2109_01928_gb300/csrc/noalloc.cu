@@ -28,7 +28,7 @@ namespace {
 constexpr size_t SCRATCH_BYTES = DEBYE_NOALLOC_SCRATCH_BYTES;
 constexpr int MAX_UNITS = 4096;
 constexpr int MAX_DEVICES = 64;
-// every sample takes 64 B of the scratch (two float4 records in kf32 and in kff)
+// every sample takes 64 B of the scratch (three float4 records; 16 B are spare)
 constexpr int64_t MAX_SAMPLES = (int64_t)(SCRATCH_BYTES / (4 * sizeof(float4)));
 
 static __device__ __align__(256) unsigned char g_scratch[SCRATCH_BYTES];
@@ -224,8 +224,8 @@ extern "C" int debye_eval_population_noalloc(const debye_options* opt_in, const 
   const int npk = nm1 * (nm1 + 1) / 2;
   int* status = (int*)cv.take(sizeof(int));
   Unit* d_units = (Unit*)cv.take(sizeof(Unit) * n_units);
-  float4* kf32 = (float4*)cv.take(sizeof(float4) * 2 * n_samples);
-  float4* kff = (float4*)cv.take(sizeof(float4) * 2 * n_samples);
+  float4* kqa = (float4*)cv.take(sizeof(float4) * 2 * n_samples);   // sample planes 0 and 1
+  float4* kqb = (float4*)cv.take(sizeof(float4) * 2 * n_samples);   // plane 2, then the granules
   double* h0 = (double*)cv.take(sizeof(double) * 2 * S);   // sum eps', then b^T b
   Scratch sc{};
   sc.Q = Q;
@@ -249,6 +249,11 @@ extern "C" int debye_eval_population_noalloc(const debye_options* opt_in, const 
     return DEBYE_EINVAL;
   }
 
+  // The granules (mixed precision) take plane 3's place; with hardly more samples than
+  // spectra they do not fit there (n / 32 + S > n, so 16.6 B per spectrum at most) and take
+  // the factor's (24 B per candidate at least), which only the FP64 path uses.
+  float4* kg = granule_count(n_samples, S) <= n_samples ? kqb + n_samples : (float4*)sc.L;
+
   int sms = 1;
   int dev = 0;
   cudaGetDevice(&dev);
@@ -260,17 +265,17 @@ extern "C" int debye_eval_population_noalloc(const debye_options* opt_in, const 
     cudaGetLastError();
     return fail_msg(DEBYE_ECUDA, err, err_len, cudaGetErrorString(e));
   }
-  launch_prep(n_samples, S, sp->offsets, sp->omega, sp->eps_re, sp->eps_im, sp->lo, sp->hi, kf32, kff, h0,
-              status, sms, st);
+  launch_prep(n_samples, S, sp->offsets, sp->omega, sp->eps_re, sp->eps_im, sp->lo, sp->hi, kqa,
+              kqa + n_samples, kqb, kg, h0, status, sms, st);
 
   EvalArgs a{};
   a.units = d_units;
   a.n_units = n_units;
   a.theta = theta;
-  a.kf32 = kf32;
-  a.kff = kff;
-  a.kq32 = kf32 + n_samples;
-  a.kqff = kff + n_samples;
+  a.kq0 = kqa;
+  a.kq1 = kqa + n_samples;
+  a.kq2 = kqb;
+  a.kg = kg;
   a.omega = sp->omega;
   a.eps_re = sp->eps_re;
   a.eps_im = sp->eps_im;

@@ -11,15 +11,14 @@ namespace debyefit {
 // Gram, residual and gradient passes the FP64 path.
 template <int N>
 void launch_pass_n(int phase, const EvalArgs& a, int grid, int block, cudaStream_t st) {
-  // the cost-only column-sum pass up to 12 poles fits in 168 registers without
-  // spills: cap it for 3 resident 128-thread blocks; larger N, the gradient
-  // variant and the FP64 passes keep the full register file (one sweep over the
-  // samples keeps a lone active lane's latency low in masked evaluations)
-  constexpr int MB_SUMS = N <= 12 ? 3 : 1;
+  // the column-sum pass sweeps at most SQUARED_CHUNK poles at a time, which fits 168
+  // registers (3 resident 128-thread blocks; 4 blocks, 128 registers: N = 12 1.109 ms
+  // against 1.065 ms); with the derivative sums 2 blocks
+  constexpr int MB_SUMS = 3, MB_SUMSG = 2;
   constexpr int MAXT = N <= 12 ? 128 : 256;
   switch (phase) {
-    case PH_SUMS: k_pass_sums<N, false, MAXT, MB_SUMS><<<grid, block, 0, st>>>(a); break;
-    case PH_SUMSG: k_pass_sums<N, true, MAXT, 1><<<grid, block, 0, st>>>(a); break;
+    case PH_SUMS: k_pass_sums<N, false, MAX_BLOCK, MB_SUMS><<<grid, block, 0, st>>>(a); break;
+    case PH_SUMSG: k_pass_sums<N, true, MAX_BLOCK, MB_SUMSG><<<grid, block, 0, st>>>(a); break;
     case PH_GRAM: k_pass<PH_GRAM, N, N, MAXT, 1><<<grid, block, 0, st>>>(a); break;
     case PH_GRAM_SUMS: k_pass<PH_GRAM_SUMS, N, N, MAXT, 1><<<grid, block, 0, st>>>(a); break;
     case PH_REFINE: k_pass<PH_REFINE, N, N, MAXT, 1><<<grid, block, 0, st>>>(a); break;

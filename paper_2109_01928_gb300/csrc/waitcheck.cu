@@ -9,7 +9,7 @@
 namespace debyefit {
 
 __global__ void k_stage_wait_check(EvalArgs a, int* waited_ok) {
-  __shared__ __align__(128) float4 stage_buf[4 * STAGE_SAMPLES];
+  __shared__ __align__(128) float4 stage_buf[STAGE_RECORDS];
   __shared__ __align__(8) uint64_t stage_bar[2];
   Stage st;
   stage_init(st, stage_buf, stage_bar);
