@@ -25,9 +25,17 @@ void launch_pass_n(int phase, const EvalArgs& a, int grid, int block, cudaStream
     case PH_SOLVE:
     case PH_SOLVEG:
       if constexpr (N <= SOLVE_N_MAX) {   // one thread per candidate (block = candidates per unit)
-        const size_t smem = solve_smem_per_thread(N) * block;   // <= 46.6 KB (N = 12, 128 threads)
-        if (phase == PH_SOLVE) k_solve_sums_t<N, 0><<<grid, block, smem, st>>>(a, a.out_cost, a.out_weights, nullptr);
-        else k_solve_sums_t<N, 1><<<grid, block, smem, st>>>(a, a.out_cost, a.out_weights, a.out_grad);
+        if constexpr (N >= SOLVE_ROLL_FROM) {
+          const int slices = block / 32, g = std::min(grid * slices, a.n_units * slices);
+          if (phase == PH_SOLVE)
+            k_solve_rows<N, 0><<<g, 32, solve_roll_bytes(N), st>>>(a, slices, a.out_cost, a.out_weights, nullptr);
+          else
+            k_solve_rows<N, 1><<<g, 32, solve_roll_bytes(N), st>>>(a, slices, a.out_cost, a.out_weights, a.out_grad);
+        } else if (phase == PH_SOLVE) {
+          k_solve_sums_t<N, 0><<<grid, block, 0, st>>>(a, a.out_cost, a.out_weights, nullptr);
+        } else {
+          k_solve_sums_t<N, 1><<<grid, block, 0, st>>>(a, a.out_cost, a.out_weights, a.out_grad);
+        }
       }
       break;
     default: k_pass<PH_GRAD, N, N, MAXT, 1><<<grid, block, 0, st>>>(a); break;
