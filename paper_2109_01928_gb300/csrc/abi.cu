@@ -233,6 +233,7 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, cudaStream_
   an.eps_re = sp->eps_re;
   an.eps_im = sp->eps_im;
   an.ks = KSN;
+  an.sums_f64 = 1;   // the coefficients are formed in FP64
   an.lam = opt.lam_search;
   an.sc.Q = qn;
   an.sc.nmax = TAB_NODE_N;

@@ -53,10 +53,12 @@ struct Scratch {
   int64_t Q;        // candidates in this evaluation (SoA stride)
   int32_t nmax;     // pole capacity of theta / weights rows
   int32_t ng;       // per-candidate Gram record: packed (nmax+1) lower triangle + h
-  double* G;        // [ng][Q]   Gram (packed) followed by h = A^T b
+  double* G;        // [ng][Q]   Gram (packed) followed by h = A^T b; mixed precision: the column
+                    //           sums S, h (and D, E), [N][Q] each, in float-float (float2)
   double* L;        // [npk][Q]  Cholesky factor of the scaled damped matrix
   double* dinv;     // [nmax+1][Q] 1 / sqrt(G_ii)
-  double* x;        // [nmax+1][Q] current (unflipped) weights
+  double* x;        // [nmax+1][Q] current (unflipped) weights; mixed precision: tau [N][Q] in
+                    //           float-float (float2)
   double* xh;       // [nmax+1][Q] flipped weights
   double* w;        // [nmax+1][Q] adjoint solve M^-1 S g_hat (gradient only)
   double* rt;       // [nmax+2][Q] rr = ||r||^2 then t = A^T r
@@ -117,6 +119,7 @@ struct EvalArgs {
   const uint8_t* active;   // [Q] optional candidate mask (nullptr: all)
   int32_t* n_failed;       // [S] optional: +1 per evaluated candidate whose damped matrix is not
                            //   positive definite (its cost is +inf)
+  int32_t sums_f64;        // column-sum pass: write tau and the sums in FP64 (the tables' node pass)
   int32_t ks;              // lanes per candidate in the pass kernels (power of two <= 32)
   double lam;
   double* out_cost;        // PH_SOLVE / PH_SOLVEG outputs: cost [Q], weights [Q][nmax+1] or
@@ -153,11 +156,6 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
   float bb = __fsub_rn(s, a);
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
-__device__ __forceinline__ void split_double(double v, float& hi, float& lo) {
-  hi = __double2float_rn(v);
-  lo = __double2float_rn(v - (double)hi);
 }
 
 // ------------------------------------------------------------------ packed FP32
@@ -236,11 +234,69 @@ __device__ __forceinline__ void v_add_pos(V& ah, V& al, V xh, V xl) {
 struct ff {
   float h, l;
 };
+// Conversions between FP64 and float-float without the FP64 pipe: on this GPU every FP64
+// operation, conversions included, holds a sub-partition's FP64 pipe for 64 cycles per
+// warp, so splitting a double the plain way (two conversions to FP32, one back, one
+// subtraction) costs 260 cycles, as much as 13 float-float multiply-adds. The integer forms
+// below take about 15 instructions and give the same bits; values outside the stated
+// exponent ranges (zeros, subnormal and huge values, infinities, NaN) take the plain way.
+//
+// (h, l): h the FP32 nearest v, l the FP32 nearest v - h.
 __device__ __forceinline__ ff ff_of(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const uint32_t e = (hi >> 20) & 0x7ffu;
   ff r;
-  r.h = __double2float_rn(v);
-  r.l = __double2float_rn(v - (double)r.h);
+  if (e - (1023u - 70u) <= 180u) {   // 2^-70 <= |v| < 2^111: every part is a normal FP32 value
+    const uint32_t sign = hi & 0x80000000u;
+    // round the 52-bit fraction to 23 bits, ties to even (the carry may reach the exponent)
+    const uint64_t rb = (((uint64_t)hi << 32) | lo) + (0x0fffffffu + ((lo >> 29) & 1u));
+    const uint32_t rlo = (uint32_t)rb, rhi = (uint32_t)(rb >> 32);
+    r.h = __uint_as_float((__funnelshift_r(rlo, rhi, 29) - (896u << 23)) | sign);   // rebiased exponent
+    // the remainder in units of 2^(exponent - 52), below 2^28 in magnitude
+    const int d = (int)(lo - (rlo & 0xe0000000u));
+    const uint32_t unit = (((hi & 0x7ff00000u) << 3) - (948u << 23)) | sign;
+    r.l = __fmul_rn(__int2float_rn(d), __uint_as_float(unit));
+  } else {
+    r.h = __double2float_rn(v);
+    r.l = __double2float_rn(v - (double)r.h);
+  }
   return r;
+}
+// Entry i of a float-float scratch array (Scratch::x and Scratch::G in mixed precision).
+__device__ __forceinline__ ff load_ff(const double* p, int64_t i) {
+  const float2 v = reinterpret_cast<const float2*>(p)[i];
+  return ff{v.x, v.y};
+}
+__device__ __forceinline__ void store_ff(double* p, int64_t i, ff v) {
+  reinterpret_cast<float2*>(p)[i] = make_float2(v.h, v.l);
+}
+// A non-negative integer up to 2^30.
+__device__ __forceinline__ ff ff_of_int(int v) {
+  const float h = __int2float_rn(v);
+  return ff{h, __int2float_rn(v - (int)h)};
+}
+// The FP64 value of an FP32 one.
+__device__ __forceinline__ double dbl_of(float a) {
+  const uint32_t b = __float_as_uint(a), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)   // normal
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + (896u << 20))), (int)(b << 29));
+  return m == 0 ? __hiloint2double((int)b, 0) : (double)a;
+}
+// ff_of((double)a.h + (double)a.l) of a normalised a: the low part rounded to the last bit
+// of the sum's FP64 value, by adding and removing a power of two whose last bit that is.
+__device__ __forceinline__ ff ff_round53(ff a) {
+  const uint32_t hb = __float_as_uint(a.h), lb = __float_as_uint(a.l);
+  uint32_t e = hb & 0x7f800000u;
+  if (e - (60u << 23) < (190u << 23)) {   // 2^-67 <= |h| < 2^123
+    if ((hb & 0x007fffffu) == 0 && (int)(hb ^ lb) < 0 && a.l != 0.f) e -= 1u << 23;   // the sum lies below a power of two
+    const float c = __uint_as_float((e - (29u << 23)) | (lb & 0x80000000u));
+    if (fabsf(a.l) < fabsf(c)) a.l = __fsub_rn(__fadd_rn(a.l, c), c);
+    return a;
+  }
+  const double v = (double)a.h + (double)a.l;
+  a.h = __double2float_rn(v);
+  a.l = __double2float_rn(v - (double)a.h);
+  return a;
 }
 __device__ __forceinline__ double ff_dbl(ff a) { return (double)a.h + (double)a.l; }
 __device__ __forceinline__ ff ff_sum(ff a, ff b) {

@@ -376,7 +376,8 @@ __device__ __forceinline__ bool stage_wait(const EvalArgs& a, Stage& st, int b) 
 // Fast2Sum is exact; the bias is removed at the end. Writes tau_i = 10^theta_i to
 // sc.x[i Q + q] (the FP64 power is done once per candidate here rather than again
 // in the solve), sc.G[i Q + q] = S_i, sc.G[(N + i) Q + q] = h_i, and with GRAD
-// sc.G[(2N + i) Q + q] = D_i, sc.G[(3N + i) Q + q] = E_i.
+// sc.G[(2N + i) Q + q] = D_i, sc.G[(3N + i) Q + q] = E_i: in float-float, as the solves
+// read them.
 //
 // The steps of one pole (V = float) or of a pair of poles (V = float2).
 template <class V, bool GRAD>
@@ -445,7 +446,9 @@ __device__ __forceinline__ float& v_half(float& v, int) { return v; }
 static __device__ __noinline__ double sums_tau(double theta, float& h, float& l) {
   const double tau = exp10(theta);
   const double ts = tau * 0x1p30;
-  split_double(ts * ts, h, l);
+  const ff t2 = ff_of(ts * ts);
+  h = t2.h;
+  l = t2.l;
   return tau;
 }
 
@@ -478,25 +481,46 @@ struct PoleSums {
       group_sum_ff(wh, wl, ks);
     }
   }
-  // S, h (and D, E) of pole j of candidate q in FP64
-  template <int N>
-  __device__ __forceinline__ void write(const EvalArgs& a, int q, int j, int ks) const {
-    double* G = a.sc.G;
-    const int64_t Q = a.sc.Q;
-    constexpr double LN10 = 2.302585092994046;
-    const double tau = a.sc.x[(int64_t)j * Q + q];
-    const double B = (double)ch + (double)cl;
-    G[(int64_t)j * Q + q] = ((double)sh - (double)ks) + (double)sl;
-    G[(int64_t)(N + j) * Q + q] = ((double)ah + (double)al) + tau * B;
+};
+
+// S, h (and D, E) of one pole in FP64, stored in float-float with tau (or as they are:
+// sums_f64): tau at x[0], the sums at G[0], G[dn], G[2 dn], G[3 dn]. One copy of the code
+// per kernel, called for every pole.
+template <bool GRAD>
+static __device__ __noinline__ void sums_write(double* x, double* G, int64_t dn, PoleSums<GRAD> s, int ks,
+                                               bool sums_f64) {
+  constexpr double LN10 = 2.302585092994046;
+  const double tau = x[0];
+  const double B = dbl_of(s.ch) + dbl_of(s.cl);
+  const double h = (dbl_of(s.ah) + dbl_of(s.al)) + tau * B;
+  // the bias is removed exactly (sh >= ks); the sum's FP64 rounding is that of its low part
+  ff S;
+  two_sum(__fsub_rn(s.sh, (float)ks), s.sl, S.h, S.l);
+  double D = 0.0, E = 0.0;
+  if constexpr (GRAD) {
+    const double U = dbl_of(__fsub_rn(s.uh, (float)ks)) + dbl_of(s.ul);
+    const double Vs = dbl_of(s.vh) + dbl_of(s.vl);
+    const double W = dbl_of(s.wh) + dbl_of(s.wl);
+    D = -2.0 * LN10 * U;
+    E = LN10 * (-2.0 * Vs + tau * (B - 2.0 * W));
+  }
+  if (sums_f64) {
+    G[0] = dbl_of(S.h) + dbl_of(S.l);
+    G[dn] = h;
     if constexpr (GRAD) {
-      const double U = ((double)uh - (double)ks) + (double)ul;
-      const double Vs = (double)vh + (double)vl;
-      const double W = (double)wh + (double)wl;
-      G[(int64_t)(2 * N + j) * Q + q] = -2.0 * LN10 * U;
-      G[(int64_t)(3 * N + j) * Q + q] = LN10 * (-2.0 * Vs + tau * (B - 2.0 * W));
+      G[2 * dn] = D;
+      G[3 * dn] = E;
+    }
+  } else {
+    store_ff(x, 0, ff_of(tau));
+    store_ff(G, 0, ff_round53(S));
+    store_ff(G, dn, ff_of(h));
+    if constexpr (GRAD) {
+      store_ff(G, 2 * dn, ff_of(D));
+      store_ff(G, 3 * dn, ff_of(E));
     }
   }
-};
+}
 
 // Every product that a granule adds to the sums of half k of t is at most the accumulator
 // it is added to: re <= 1 / (1 + w2min tau^2) and u = re (1 - re) <= min(re, 1/4, x^2) up
@@ -623,7 +647,10 @@ __device__ __forceinline__ bool sums_sq_sweep(const EvalArgs& a, const Unit& u, 
     if (own == ln.slice) mine = t;
     if (own == ln.ks - 1 || i == C - 1) {
       const int k = i - own + ln.slice;   // this lane's pole of the group's last ks poles
-      if (ln.act && k < C) mine.template write<N>(a, q, P0 + k, ln.ks);
+      if (ln.act && k < C) {
+        const int64_t at = (int64_t)(P0 + k) * a.sc.Q + q;
+        sums_write<GRAD>(a.sc.x + at, a.sc.G + at, N * a.sc.Q, mine, ln.ks, a.sums_f64 != 0);
+      }
     }
   }
   return true;

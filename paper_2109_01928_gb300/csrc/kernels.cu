@@ -21,14 +21,11 @@ __global__ void k_prep_samples(int64_t n, const double* __restrict__ omega,
        k += (int64_t)gridDim.x * blockDim.x) {
     const double w = omega[k], a = er[k], b = ei[k];
     if (!(w > 0.0) || !isfinite(w) || !isfinite(a) || !isfinite(b)) set_status(status, DEBYE_ENOTFINITE);
-    float h, l;
     const double ws = w * 0x1p-30;
-    split_double(ws * ws, h, l);
-    kq0[k] = make_float4(h, h, l, l);
-    split_double(a, h, l);
-    kq1[k] = make_float4(h, h, l, l);
-    split_double(w * b, h, l);
-    kq2[k] = make_float4(h, h, l, l);
+    const ff w2 = ff_of(ws * ws), e = ff_of(a), c = ff_of(w * b);
+    kq0[k] = make_float4(w2.h, w2.h, w2.l, w2.l);
+    kq1[k] = make_float4(e.h, e.h, e.l, e.l);
+    kq2[k] = make_float4(c.h, c.h, c.l, c.l);
   }
 }
 
@@ -386,7 +383,7 @@ __global__ void __launch_bounds__(WARP_SOLVE_MAX_WARPS * 32) k_solve_sums_warp(E
   for (int ui = blockIdx.x; ui < a.n_units; ui += gridDim.x) {
     const Unit u = a.units[ui];
     const int N = u.N, n = N + 1;
-    const ff kk = ff_of((double)(u.k1 - u.k0));
+    const ff kk = ff_of_int((int)(u.k1 - u.k0));
     for (int q = u.q0 + wid; q < u.q1; q += nw) {   // warp-uniform from here on
       if (a.active && !a.active[q]) continue;
       // row r >= 1 is pole r - 1: tau (from the column-sum pass), S and h
@@ -396,10 +393,10 @@ __global__ void __launch_bounds__(WARP_SOLVE_MAX_WARPS * 32) k_solve_sums_warp(E
         hv = ff_of(a.h0[u.s]);
         gd = kk;
       } else if (r < n) {
-        m.tau[r] = ff_of(a.sc.x[(int64_t)(r - 1) * Q + q]);
-        gd = ff_of(a.sc.G[(int64_t)(r - 1) * Q + q]);
+        m.tau[r] = load_ff(a.sc.x, (int64_t)(r - 1) * Q + q);
+        gd = load_ff(a.sc.G, (int64_t)(r - 1) * Q + q);
         m.S[r] = gd;
-        hv = ff_of(a.sc.G[(int64_t)(N + r - 1) * Q + q]);
+        hv = load_ff(a.sc.G, (int64_t)(N + r - 1) * Q + q);
       }
       if (r < n) m.dinv[r] = __frsqrt_rn(gd.h);
       __syncwarp();
@@ -472,8 +469,8 @@ __global__ void __launch_bounds__(WARP_SOLVE_MAX_WARPS * 32) k_solve_sums_warp(E
         double gi = 0.0;
         if (i < N) {
           const ff ln10 = ff_of(2.302585092994046);
-          const ff Di = ff_of(a.sc.G[(int64_t)(2 * N + i) * Q + q]);
-          const ff Ei = ff_of(a.sc.G[(int64_t)(3 * N + i) * Q + q]);
+          const ff Di = load_ff(a.sc.G, (int64_t)(2 * N + i) * Q + q);
+          const ff Ei = load_ff(a.sc.G, (int64_t)(3 * N + i) * Q + q);
           const ff ti = m.tau[r], Si = m.S[r];
           ff ax = ff_prod(Di, m.xh[0]), aw = ff_prod(Di, m.w[0]), as = ax;
           for (int j = 1; j < n; ++j) {

@@ -173,12 +173,12 @@ __global__ void __launch_bounds__(128) k_solve_sums_t(EvalArgs a, double* cost, 
     float L[APK], dinv[AN1], v[AN1];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      tau[i] = ff_of(a.sc.x[(int64_t)i * Q + q]);   // 10^theta_i from the column-sum pass
-      S[i] = ff_of(a.sc.G[(int64_t)i * Q + q]);
-      hv[i + 1] = ff_of(a.sc.G[(int64_t)(N + i) * Q + q]);
+      tau[i] = load_ff(a.sc.x, (int64_t)i * Q + q);   // 10^theta_i from the column-sum pass
+      S[i] = load_ff(a.sc.G, (int64_t)i * Q + q);
+      hv[i + 1] = load_ff(a.sc.G, (int64_t)(N + i) * Q + q);
     }
     hv[0] = ff_of(a.h0[u.s]);
-    const ff kk = ff_of((double)(u.k1 - u.k0));
+    const ff kk = ff_of_int((int)(u.k1 - u.k0));
     const ff one_lam = ff_of(1.0 + a.lam);
     // the general kernel's gradient variant keeps the entries in a table: its five
     // products with M outweigh the table's local-memory traffic (measured on N = 20:
@@ -254,8 +254,8 @@ __global__ void __launch_bounds__(128) k_solve_sums_t(EvalArgs a, double* cost, 
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const int I = i + 1;
-      const ff Di = ff_of(a.sc.G[(int64_t)(2 * N + i) * Q + q]);
-      const ff Ei = ff_of(a.sc.G[(int64_t)(3 * N + i) * Q + q]);
+      const ff Di = load_ff(a.sc.G, (int64_t)(2 * N + i) * Q + q);
+      const ff Ei = load_ff(a.sc.G, (int64_t)(3 * N + i) * Q + q);
       // row i of M_i against x_hat, w and x* (x*_j = s_j x_hat_j), off the diagonal
       ff ax = ff_prod(Di, x[0]), aw = ff_prod(Di, w[0]), as = ax;
 #pragma unroll
@@ -428,10 +428,10 @@ __global__ void __launch_bounds__(32) k_solve_rows(EvalArgs a, int slices, doubl
       set_status(a.status, DEBYE_EBOUNDS);
       continue;
     }
-    auto tau_of = [&](int i) { return ff_of(a.sc.x[(int64_t)i * Q + q]); };
-    auto S_of = [&](int i) { return ff_of(a.sc.G[(int64_t)i * Q + q]); };
+    auto tau_of = [&](int i) { return load_ff(a.sc.x, (int64_t)i * Q + q); };
+    auto S_of = [&](int i) { return load_ff(a.sc.G, (int64_t)i * Q + q); };
     const ff one_lam = ff_of(1.0 + a.lam);
-    const ff kk = ff_of((double)(u.k1 - u.k0));
+    const ff kk = ff_of_int((int)(u.k1 - u.k0));
     float dinv[n];
     M.put(0, ff_prod(kk, one_lam));
     dinv[0] = __frsqrt_rn(kk.h);
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(32) k_solve_rows(EvalArgs a, int slices, doubl
     ff hv[n], x[n];
     hv[0] = ff_of(a.h0[u.s]);
 #pragma unroll
-    for (int i = 0; i < N; ++i) hv[i + 1] = ff_of(a.sc.G[(int64_t)(N + i) * Q + q]);
+    for (int i = 0; i < N; ++i) hv[i + 1] = load_ff(a.sc.G, (int64_t)(N + i) * Q + q);
     if (ok) ok = refined_solve_rows<n>(L, dinv, M, R, hv, x, GRAD ? SUMS_REFINE : SUMS_REFINE_COST);
     record_fail(a, q, u.s, ok);
     if (!ok) {
@@ -530,8 +530,8 @@ __global__ void __launch_bounds__(32) k_solve_rows(EvalArgs a, int slices, doubl
       for (int i = 0; i < N; ++i) {
         const int I = i + 1;
         const ff ti = tau_of(i), Si = S_of(i);
-        const ff Di = ff_of(a.sc.G[(int64_t)(2 * N + i) * Q + q]);
-        const ff Ei = ff_of(a.sc.G[(int64_t)(3 * N + i) * Q + q]);
+        const ff Di = load_ff(a.sc.G, (int64_t)(2 * N + i) * Q + q);
+        const ff Ei = load_ff(a.sc.G, (int64_t)(3 * N + i) * Q + q);
         // row i of M_i against x_hat, w and x* (x*_j = s_j x_hat_j), off the diagonal
         ff ax = ff_prod(Di, x[0]), aw = ff_prod(Di, w[0]), as = ax;
 #pragma unroll

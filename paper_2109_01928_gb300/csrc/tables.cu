@@ -157,9 +157,33 @@ __device__ void direct_sums(const EvalArgs& a, const Unit& u, double tau, double
   out[3] = LN10 * (-2.0 * V + tau * (C - 2.0 * W));
 }
 
+// Segment of position uu (in segments from the table's origin), or -1 outside [0, ns]:
+// the integer part from the bits of uu (the FP64 comparisons and conversions would each
+// hold the FP64 pipe for 64 cycles per warp).
+__device__ __forceinline__ int tab_segment(double uu, int ns) {
+  const uint32_t hi = (uint32_t)__double2hiint(uu), lo = (uint32_t)__double2loint(uu);
+  if (((hi << 1) | lo) == 0) return 0;   // +-0
+  const int e = (int)(hi >> 20) - 1023;  // sign set: beyond every bound
+  if (e < 0) return 0;
+  if (e > 10) return -1;                 // 2048 and more (TAB_MAX_SEG is 1000), negative, infinite or NaN
+  const uint32_t m = (hi & 0xfffffu) | 0x100000u;
+  const int g = (int)(m >> (20 - e));
+  if (g < ns) return g;
+  return g == ns && ((m << (12 + e)) | lo) == 0 ? ns - 1 : -1;   // the upper bound itself
+}
+
+// A positive integer below 2^20 as a double.
+__device__ __forceinline__ double dbl_of_int(uint32_t m) {
+  const int z = __clz((int)m);
+  return __hiloint2double((int)(((uint32_t)(1023 + 31 - z) << 20) + ((m << z << 1) >> 12)), 0);
+}
+
 // Column sums of every (candidate, pole) of the units from the tables, written where
 // the column-sum pass writes them (tau to sc.x row i; S, h, dS, dh to G rows i, N + i,
-// 2N + i, 3N + i) for the column-sum solves. One thread per (candidate, pole).
+// 2N + i, 3N + i, in float-float) for the column-sum solves. One thread per (candidate,
+// pole). With the position and the results converted by integer operations, 3 FP64
+// operations per pole are left of 20, whose pipe bound the kernel: 88 -> 67 us for 1024
+// spectra x 256 candidates, N 2-12.
 template <bool GRAD>
 __global__ void __launch_bounds__(128) k_tab_eval(EvalArgs a) {
   const int64_t Q = a.sc.Q;
@@ -175,30 +199,32 @@ __global__ void __launch_bounds__(128) k_tab_eval(EvalArgs a) {
       if (a.active && !a.active[q]) continue;
       const double th = a.theta[(int64_t)q * a.sc.nmax + j];
       const double d = th - l;
-      const double uu = d * TAB_INV_W;
-      double tau, v[4] = {0.0, 0.0, 0.0, 0.0};
-      if (uu >= 0.0 && uu <= (double)ns) {
-        // x = 2 (uu - g) - 1 in [-1, 1]; the FP64 work stays a handful of operations
-        const int g = min((int)uu, ns - 1);
-        const ff x = ff_of(fma(d, 2.0 * TAB_INV_W, -(double)(2 * g + 1)));
+      const int g = tab_segment(d * TAB_INV_W, ns);
+      ff tau, v[4];
+      if (g >= 0) {
+        // x = 2 (uu - g) - 1 in [-1, 1]
+        const ff x = ff_of(fma(d, 2.0 * TAB_INV_W, -dbl_of_int(2 * g + 1)));
         const float2* c = cs + (int64_t)g * (TAB_NF * TAB_NC);
-        v[0] = ff_dbl(poly_ff(c, x));
-        v[1] = ff_dbl(poly_ff(c + TAB_NC, x));
-        tau = ff_dbl(poly_ff(c + 2 * TAB_NC, x));
+        v[0] = ff_round53(poly_ff(c, x));
+        v[1] = ff_round53(poly_ff(c + TAB_NC, x));
+        tau = ff_round53(poly_ff(c + 2 * TAB_NC, x));
         if (GRAD) {
-          v[2] = ff_dbl(poly_ff(c + 3 * TAB_NC, x));
-          v[3] = ff_dbl(poly_ff(c + 4 * TAB_NC, x));
+          v[2] = ff_round53(poly_ff(c + 3 * TAB_NC, x));
+          v[3] = ff_round53(poly_ff(c + 4 * TAB_NC, x));
         }
       } else {
-        tau = exp10(th);
-        direct_sums<GRAD>(a, u, tau, v);
+        double s[4];
+        const double t = exp10(th);
+        direct_sums<GRAD>(a, u, t, s);
+        tau = ff_of(t);
+        for (int f = 0; f < (GRAD ? 4 : 2); ++f) v[f] = ff_of(s[f]);
       }
-      a.sc.x[(int64_t)j * Q + q] = tau;
-      G[(int64_t)j * Q + q] = v[0];
-      G[(int64_t)(N + j) * Q + q] = v[1];
+      store_ff(a.sc.x, (int64_t)j * Q + q, tau);
+      store_ff(G, (int64_t)j * Q + q, v[0]);
+      store_ff(G, (int64_t)(N + j) * Q + q, v[1]);
       if (GRAD) {
-        G[(int64_t)(2 * N + j) * Q + q] = v[2];
-        G[(int64_t)(3 * N + j) * Q + q] = v[3];
+        store_ff(G, (int64_t)(2 * N + j) * Q + q, v[2]);
+        store_ff(G, (int64_t)(3 * N + j) * Q + q, v[3]);
       }
     }
   }
