@@ -408,14 +408,13 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
   if (mixed) {
     // one float-float column-sum pass (with the derivative sums when the gradient is
     // wanted), then weights, cost and gradient from the exact Gram identity of the
-    // Debye columns. With the thread-per-candidate solve, buckets up to SOLVE_N_MAX
-    // poles solve in a per-N kernel (systems in registers) launched right after the
-    // bucket's pass on the bucket's stream; the other buckets take the general
-    // kernel after the join, and the warp-per-candidate solve runs after it. With
-    // kernel timing on, the per-N solves run after the timed pass, timed on their own.
+    // Debye columns. With the thread-per-candidate solve every bucket's solve is
+    // launched right after the bucket's pass on the bucket's stream; the
+    // warp-per-candidate solve runs after the join. With kernel timing on, the per-N
+    // solves run after the timed pass, timed on their own.
     const int ph = grad ? PH_SUMSG : PH_SUMS, sph = grad ? PH_SOLVEG : PH_SOLVE;
     const bool by_warp = solve_sums_by_warp(a.sc.Q, opt.solve_lanes, sms);
-    const int nb_n = by_warp ? 0 : SOLVE_N_MAX;   // buckets with a per-N solve
+    const int nb_n = by_warp ? 0 : N_BUCKETS;   // buckets with a per-N solve
     auto solve_bucket = [&](int b, const EvalArgs& ab, cudaStream_t bs) {
       if (b >= nb_n) return;
       EvalArgs as = ab;
@@ -440,16 +439,7 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
       if (!rc) rc = fork_buckets(DEBYE_KERNEL_SOLVE, 0.0, nb_n, solve_bucket);
     }
     if (rc) return rc;
-    const int u0 = g.begin[nb_n], rest = g.begin[N_BUCKETS] - u0;
-    if (rest) {
-      EvalArgs ar = a;
-      ar.units = a.units + u0;
-      ar.n_units = rest;
-      timed(DEBYE_KERNEL_SOLVE, [&] {
-        if (by_warp) launch_solve_sums_warp(ar, cost, weights, grad, cb, sms, st);
-        else launch_solve_sums(ar, cost, weights, grad, gblock, sms, st);
-      });
-    }
+    if (by_warp) timed(DEBYE_KERNEL_SOLVE, [&] { launch_solve_sums_warp(a, cost, weights, grad, cb, sms, st); });
     return check_launch("column-sum solve");
   }
   if ((rc = per_bucket(opt.precision == DEBYE_PREC_FP64_SUMS ? PH_GRAM_SUMS : PH_GRAM))) return rc;

@@ -27,9 +27,6 @@ enum Phase { PH_GRAM = 0, PH_REFINE = 1, PH_GRAD = 2, PH_SUMS = 3, PH_SUMSG = 4,
              PH_SOLVE = 5, PH_SOLVEG = 6,
              // FP64 column sums and the Gram from the partial-fraction identity (FP64 path)
              PH_GRAM_SUMS = 7 };
-// Largest pole count with a compile-time (register-resident) column-sum solve;
-// larger ones use the general kernel.
-constexpr int SOLVE_N_MAX = 12;
 // The column-sum pass (eval.cuh) sweeps the samples for at most this many poles at a time
 // (8 registers per pole, 14 with the derivative sums), two samples per step: measured on
 // 128 spectra x 512 candidates x 1024 samples at 64 candidates x 2 lanes, N = 12 0.941 ms

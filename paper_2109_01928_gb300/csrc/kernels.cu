@@ -593,15 +593,6 @@ static int grid_for(int n_units, int sms, int per_sm) {
   return std::max(1, std::min(n_units, sms * per_sm));
 }
 
-// One thread per candidate with per-thread arrays in local memory: a grid of up to
-// 32 blocks per SM keeps enough warps resident to hide that memory's latency.
-void launch_solve_sums(const EvalArgs& a, double* cost, double* weights, double* grad, int block, int sms,
-                       cudaStream_t st) {
-  if (!a.n_units) return;
-  if (grad) k_solve_sums_t<0, 1><<<grid_for(a.n_units, sms, 32), block, 0, st>>>(a, cost, weights, grad);
-  else k_solve_sums_t<0, 0><<<grid_for(a.n_units, sms, 32), block, 0, st>>>(a, cost, weights, nullptr);
-}
-
 bool solve_sums_by_warp(int64_t Q, int lanes, int sms) {
   if (lanes == 1 || lanes == 32) return lanes == 32;
   return Q <= (int64_t)sms * WARP_SOLVE_MAX_Q_PER_SM;

@@ -72,14 +72,12 @@ void launch_prep(int64_t n_samples, int64_t S, const int64_t* offsets, const dou
                  const double* er, const double* ei, const double* lo, const double* hi,
                  float4* kq0, float4* kq1, float4* kq2, float4* kg, double* h0, int* status, int sms,
                  cudaStream_t st);
-// Mixed evaluation after the column-sum pass: weights, flip, cost and (grad != nullptr,
-// after the pass with derivative sums) the gradient in theta.
-void launch_solve_sums(const EvalArgs& a, double* cost, double* weights, double* grad, int block, int sms,
-                       cudaStream_t st);
-// The same with one warp per candidate (lane r: row r of the small systems), for
-// evaluations too small to fill the GPU one thread per candidate. solve_sums_by_warp
-// picks it: lanes 1 or 32 force a kernel, 0 takes the warp kernel when the
-// evaluation has at most 256 candidates per SM.
+// Mixed evaluation after the column-sum pass, weights, flip, cost and (grad != nullptr,
+// after the pass with derivative sums) the gradient in theta, with one warp per candidate
+// (lane r: row r of the small systems), for evaluations too small to fill the GPU one
+// thread per candidate (PH_SOLVE, PH_SOLVEG of launch_pass). solve_sums_by_warp picks it:
+// lanes 1 or 32 force a kernel, 0 takes the warp kernel when the evaluation has at most
+// 256 candidates per SM.
 bool solve_sums_by_warp(int64_t Q, int lanes, int sms);
 void launch_solve_sums_warp(const EvalArgs& a, double* cost, double* weights, double* grad, int cands_per_unit,
                             int sms, cudaStream_t st);

@@ -295,13 +295,15 @@ extern "C" int debye_eval_population_noalloc(const debye_options* opt_in, const 
       ab.units = a.units + begin[b];
       ab.n_units = n;
       const int grid = std::max(1, std::min(n, sms * 16));
-      launch_pass(b + 1, phase, ab, grid, cb * ks, st);
+      launch_pass(b + 1, phase, ab, grid, phase == PH_SOLVE ? warp_round(cb) : cb * ks, st);
     }
   };
   if (mixed) {
     // one float-float column-sum pass, weights and cost from the exact Gram identity
     per_bucket(PH_SUMS);
-    launch_solve_sums(a, cost, weights, nullptr, warp_round(cb), sms, st);
+    a.out_cost = cost;
+    a.out_weights = weights;
+    per_bucket(PH_SOLVE);
   } else {
     per_bucket(opt.precision == DEBYE_PREC_FP64_SUMS ? PH_GRAM_SUMS : PH_GRAM);
     launch_solve(a, warp_round(cb), sms, st);

@@ -7,7 +7,7 @@
 namespace debyefit {
 
 // The column-sum passes (PH_SUMS, PH_SUMSG) and the per-N column-sum solves
-// (PH_SOLVE, PH_SOLVEG, N <= SOLVE_N_MAX) are the mixed-precision path; the
+// (PH_SOLVE, PH_SOLVEG) are the mixed-precision path; the
 // Gram, residual and gradient passes the FP64 path.
 template <int N>
 void launch_pass_n(int phase, const EvalArgs& a, int grid, int block, cudaStream_t st) {
@@ -24,18 +24,19 @@ void launch_pass_n(int phase, const EvalArgs& a, int grid, int block, cudaStream
     case PH_REFINE: k_pass<PH_REFINE, N, N, MAXT, 1><<<grid, block, 0, st>>>(a); break;
     case PH_SOLVE:
     case PH_SOLVEG:
-      if constexpr (N <= SOLVE_N_MAX) {   // one thread per candidate (block = candidates per unit)
-        if constexpr (N >= SOLVE_ROLL_FROM) {
-          const int slices = block / 32, g = std::min(grid * slices, a.n_units * slices);
-          if (phase == PH_SOLVE)
-            k_solve_rows<N, 0><<<g, 32, solve_roll_bytes(N), st>>>(a, slices, a.out_cost, a.out_weights, nullptr);
-          else
-            k_solve_rows<N, 1><<<g, 32, solve_roll_bytes(N), st>>>(a, slices, a.out_cost, a.out_weights, a.out_grad);
-        } else if (phase == PH_SOLVE) {
-          k_solve_sums_t<N, 0><<<grid, block, 0, st>>>(a, a.out_cost, a.out_weights, nullptr);
-        } else {
-          k_solve_sums_t<N, 1><<<grid, block, 0, st>>>(a, a.out_cost, a.out_weights, a.out_grad);
-        }
+      if constexpr (N >= SOLVE_ROLL_FROM) {   // a warp per block: `block` candidates per unit in slices of 32
+        const int slices = block / 32, g = std::min(grid, a.n_units) * slices;
+        const void* k = phase == PH_SOLVE ? (const void*)k_solve_rows<N, 0> : (const void*)k_solve_rows<N, 1>;
+        if constexpr (solve_roll_bytes(N) > 48 * 1024)   // set with every launch: the attribute goes with the context
+          cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_roll_bytes(N));
+        if (phase == PH_SOLVE)
+          k_solve_rows<N, 0><<<g, 32, solve_roll_bytes(N), st>>>(a, slices, a.out_cost, a.out_weights, nullptr);
+        else
+          k_solve_rows<N, 1><<<g, 32, solve_roll_bytes(N), st>>>(a, slices, a.out_cost, a.out_weights, a.out_grad);
+      } else if (phase == PH_SOLVE) {         // one thread per candidate
+        k_solve_sums_t<N, 0><<<grid, block, 0, st>>>(a, a.out_cost, a.out_weights, nullptr);
+      } else {
+        k_solve_sums_t<N, 1><<<grid, block, 0, st>>>(a, a.out_cost, a.out_weights, a.out_grad);
       }
       break;
     default: k_pass<PH_GRAD, N, N, MAXT, 1><<<grid, block, 0, st>>>(a); break;

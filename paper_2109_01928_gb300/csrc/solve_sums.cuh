@@ -33,19 +33,13 @@ __device__ __forceinline__ ff gram_ff(int i, int j, const ff* tau, const ff* S, 
   return ff_quot(num, ff_sum(tau[i - 1], tau[j - 1]));
 }
 
-// Sources of the float-float Gram entries (i >= j): formed where they are used
-// (the per-N kernels, whose compiler keeps what fits), or read from a per-thread
-// packed table filled once (the general kernel, whose arrays are in local memory
-// anyway).
+// The float-float Gram entries (i >= j), formed where they are used (the compiler keeps
+// what fits).
 struct GramRecompute {
   const ff* tau;
   const ff* S;
   ff kk;
   __device__ __forceinline__ ff operator()(int i, int j) const { return gram_ff(i, j, tau, S, kk); }
-};
-struct GramTable {
-  const ff* g;   // packed lower triangle, entry (i, j) at pk(i, j)
-  __device__ __forceinline__ ff operator()(int i, int j) const { return g[pk(i, j)]; }
 };
 
 // (M v)_i in float-float, M = G + lam diag G; each entry serves both of its rows.
@@ -149,28 +143,25 @@ __device__ __forceinline__ bool refined_solve(int n, LA L, const float* dinv, co
 //   (M_i)_{ij} = tau_i D_i / (tau_i + tau_j) + ln10 tau_i tau_j (S_i - S_j) / (tau_i + tau_j)^2
 // (the derivative of G_ij = (tau_i S_i + tau_j S_j)/(tau_i + tau_j), d tau_i = ln10 tau_i).
 //
-// NT = 0: any pole count (u.N at run time); the small systems live in per-thread
-// local memory. NT > 0 (below SOLVE_ROLL_FROM): every unit has NT poles (one launch per
-// pole bucket), the loops have constant trip counts, unroll, and the systems stay in
-// registers. GRAD (0 or 1) fixes whether the gradient is computed.
+// Every unit has NT poles (below SOLVE_ROLL_FROM; one launch per pole bucket): the loops
+// unroll and the systems stay in registers. GRAD (0 or 1) fixes whether the gradient is
+// computed.
 template <int NT, int GRAD>
 __global__ void __launch_bounds__(128) k_solve_sums_t(EvalArgs a, double* cost, double* weights, double* grad) {
   const int64_t Q = a.sc.Q;
   const int nmax = a.sc.nmax, nm1 = nmax + 1;
-  const bool with_grad = GRAD < 0 ? grad != nullptr : GRAD > 0;
+  constexpr bool with_grad = GRAD > 0;
   for (int ui = blockIdx.x; ui < a.n_units; ui += gridDim.x) {
     const Unit u = a.units[ui];
     const int q = u.q0 + (int)threadIdx.x;
     if (q >= u.q1 || (a.active && !a.active[q])) continue;
-    if (NT > 0 && u.N != NT) {
+    if (u.N != NT) {
       set_status(a.status, DEBYE_EBOUNDS);
       continue;
     }
-    const int N = NT > 0 ? NT : u.N, n = N + 1;
-    // arrays sized for the compile-time pole count (NT > 0) so that they can live in registers
-    constexpr int AN = NT > 0 ? NT : NMAX, AN1 = AN + 1, APK = AN1 * (AN1 + 1) / 2;
-    ff tau[AN], S[AN], hv[AN1], x[AN1], r[AN1];
-    float L[APK], dinv[AN1], v[AN1];
+    constexpr int N = NT, n = N + 1;
+    ff tau[N], S[N], hv[n], x[n], r[n];
+    float L[n * (n + 1) / 2], dinv[n], v[n];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       tau[i] = load_ff(a.sc.x, (int64_t)i * Q + q);   // 10^theta_i from the column-sum pass
@@ -180,20 +171,7 @@ __global__ void __launch_bounds__(128) k_solve_sums_t(EvalArgs a, double* cost, 
     hv[0] = ff_of(a.h0[u.s]);
     const ff kk = ff_of_int((int)(u.k1 - u.k0));
     const ff one_lam = ff_of(1.0 + a.lam);
-    // the general kernel's gradient variant keeps the entries in a table: its five
-    // products with M outweigh the table's local-memory traffic (measured on N = 20:
-    // cost and gradient 40.6 -> 35.5 ms; cost only, two products, 6.0 -> 7.5 ms)
-    constexpr bool G_TABLE = NT == 0 && GRAD > 0;
-    ff gtab[G_TABLE ? NPACK_MAX : 1];
-    const auto G = [&] {
-      if constexpr (!G_TABLE) {
-        return GramRecompute{tau, S, kk};
-      } else {
-        for (int i = 0; i < n; ++i)
-          for (int j = 0; j <= i; ++j) gtab[pk(i, j)] = gram_ff(i, j, tau, S, kk);
-        return GramTable{gtab};
-      }
-    }();
+    const GramRecompute G{tau, S, kk};
     // FP32 Cholesky of the Marquardt-scaled damped matrix (unit diagonal + lam)
 #pragma unroll
     for (int i = 0; i < n; ++i) dinv[i] = __frsqrt_rn(G(i, i).h);   // diag(G)^-1/2
@@ -215,7 +193,7 @@ __global__ void __launch_bounds__(128) k_solve_sums_t(EvalArgs a, double* cost, 
       continue;
     }
     // sign flip of negative d_eps (Sec. III-B), then the exact quadratic cost
-    float sgn[AN1];
+    float sgn[n];
 #pragma unroll
     for (int i = 0; i < n; ++i) {
       sgn[i] = (i > 0 && x[i].h < 0.f) ? -1.f : 1.f;
@@ -239,7 +217,7 @@ __global__ void __launch_bounds__(128) k_solve_sums_t(EvalArgs a, double* cost, 
     }
     if (!with_grad) continue;
     // adjoint w = M^-1 (s * (M x_hat - h)); r becomes its right-hand side
-    ff w[AN1], rw[AN1];
+    ff w[n], rw[n];
 #pragma unroll
     for (int i = 0; i < n; ++i) {
       r[i] = ff_sum(r[i], ff_neg(hv[i]));
@@ -300,11 +278,14 @@ __global__ void __launch_bounds__(128) k_solve_sums_t(EvalArgs a, double* cost, 
 // are in flight in the products with M: one float-float accumulation is a chain of 7
 // dependent operations per term.
 // One warp per block, one candidate per lane; element e of a lane's record at e * 32 + lane,
-// so that a warp's 8-byte accesses are contiguous: 26.6 KB per block at N = 12, 8 blocks
-// per SM. Measured on 65536 candidates, kernel timing, against the unrolled kernel: N = 12
+// so that a warp's 8-byte accesses are contiguous: 26.6 KB per block at N = 12 (8 blocks
+// per SM), 64.5 KB at N = 20 (3; the factor then spills to L1). Measured on 65536 candidates, kernel timing, against the unrolled kernel: N = 12
 // 229 -> 129 us, N = 8 75 -> 59 us, N = 4 31 -> 28 us (N = 3 equal, N = 2 slower, so the
 // line lies at 4); with the gradient N = 12 1156 -> 368 us, N = 8 296 -> 167 us, N = 4
-// 65 -> 56 us.
+// 65 -> 56 us. With tau and the sums read in float-float instead of FP64: N = 12 86 us,
+// N = 4 18 us, with the gradient 283 and 45 us. Against a general kernel with its arrays
+// in local memory: N = 20 794 -> 522 us, N = 16 475 -> 221 us, with the gradient 1963 ->
+// 1921 and 1283 -> 815 us.
 constexpr int SOLVE_ROLL_FROM = 4;
 constexpr int solve_roll_ff(int N) { return (N + 1) * (N + 2) / 2 + (N + 1); }   // M, then the product
 constexpr size_t solve_roll_bytes(int N) { return sizeof(float2) * 32 * (size_t)solve_roll_ff(N); }
