@@ -323,7 +323,35 @@ __device__ __forceinline__ ff ff_quot(ff a, ff b) {
   return ff{h, __fsub_rn(q2, __fsub_rn(h, q1))};
 }
 
-
+// 1 / d in FP64 for d >= 1 (the Debye basis's denominator): one Newton-Raphson step in
+// FP64 (two FMAs; Markstein, IBM J. Res. Dev. 34, 1990) from a float-float reciprocal good
+// to 2^-44, which the FP32 and integer pipes form and assemble into a double. The step
+// leaves 2^-88 before its rounding, so the result is the correctly rounded quotient unless
+// that lies within 2^-88 of a tie (one operand in 2^35). The division operator costs 5 times
+// 64 cycles of the FP64 pipe per warp, this 2 times. Arguments of 2^70 and more, infinite
+// or NaN, and those within 2^-20 below a power of two (whose reciprocals 1 + j 2^-53 + j^2
+// 2^-106 lie beside ties) or with the sum below in another binade take the operator.
+__device__ __forceinline__ double rcp_ge1(double d) {
+  const uint32_t hi = (uint32_t)__double2hiint(d);
+  if (hi - 0x3ff00000u < (70u << 20) && (hi & 0xfffffu) != 0xfffffu) {
+    const ff f = ff_of(d);
+    const float r0 = rcp_approx(f.h);
+    float e = __fmaf_rn(-f.h, r0, 1.0f);
+    e = __fmaf_rn(-f.l, r0, e);
+    const uint32_t rb = __float_as_uint(r0);
+    // r0 e in units of r0's last FP64 bit, below 2^31 in magnitude (rcp.approx: 1 ulp)
+    int m = __float2int_rn(__fmul_rn(__fmul_rn(r0, e), __uint_as_float((306u - (rb >> 23)) << 23)));
+    const bool pow2 = (rb & 0x007fffffu) == 0 && m < 0;   // the sum lies below a power of two: half units
+    if (pow2) m <<= 1;
+    const long long b0 = (long long)(((uint64_t)((rb >> 3) + (896u << 20)) << 32) | (rb << 29));
+    const long long b = b0 + m;
+    if (pow2 || (b ^ b0) >> 52 == 0) {
+      const double y = __longlong_as_double(b);
+      return __fma_rn(y, __fma_rn(-d, y, 1.0), y);
+    }
+  }
+  return 1.0 / d;
+}
 
 // ------------------------------------------------------------------ SplitMix64
 // Steele, Lea and Flood, "Fast splittable pseudorandom number generators",

@@ -101,7 +101,7 @@ __device__ __forceinline__ void gram_unit(const EvalArgs& a, const Unit& u) {
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const double x = w * tau[i];
-      const double r = 1.0 / fma(x, x, 1.0);
+      const double r = rcp_ge1(fma(x, x, 1.0));
       re[i] = r;
       im[i] = x * r;
     }
@@ -171,7 +171,7 @@ __device__ __forceinline__ void gram_sums_unit(const EvalArgs& a, const Unit& u)
     const double w2 = w * w;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const double r = 1.0 / fma(w2, t2[i], 1.0);
+      const double r = rcp_ge1(fma(w2, t2[i], 1.0));
       sv[i] += r;
       av[i] = fma(r, er, av[i]);
       bv[i] = fma(r, wei, bv[i]);
@@ -230,7 +230,7 @@ __device__ __forceinline__ void refine_unit(const EvalArgs& a, const Unit& u) {
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const double x = om * tau[i];
-      const double r = 1.0 / fma(x, x, 1.0);
+      const double r = rcp_ge1(fma(x, x, 1.0));
       re[i] = r;
       im[i] = x * r;
       ar = fma(-w[i], re[i], ar);
@@ -717,7 +717,7 @@ __device__ __forceinline__ void grad_unit(const EvalArgs& a, const Unit& u) {
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const double x = om * tau[i];
-      const double r = 1.0 / fma(x, x, 1.0);
+      const double r = rcp_ge1(fma(x, x, 1.0));
       xv[i] = x;
       re[i] = r;
       im[i] = x * r;

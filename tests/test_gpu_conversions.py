@@ -1,5 +1,5 @@
-"""The integer conversions between FP64 and float-float (csrc/common.cuh) and the table's
-segment lookup (csrc/tables.cu) against the plain FP64 forms, bit for bit (a zero low part
+"""The integer conversions between FP64 and float-float and the reciprocal (csrc/common.cuh)
+and the table's segment lookup (csrc/tables.cu) against the plain FP64 forms, bit for bit (a zero low part
 may differ in its sign), over random bit patterns and the edges of their ranges: powers of
 two and their neighbours, ties, carries into the exponent, zeros, subnormal and huge
 values, infinities and NaN."""
@@ -19,7 +19,7 @@ SRC = r"""
 #include "tables.cu"
 #include <cstdio>
 using namespace debyefit;
-__device__ unsigned long long bad[5];
+__device__ unsigned long long bad[6];
 __device__ bool same(float a, float b) { return __float_as_uint(a) == __float_as_uint(b) || a == b || (isnan(a) && isnan(b)); }
 __device__ bool same(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b) || (isnan(a) && isnan(b)); }
 __device__ void check_double(double v) {
@@ -67,6 +67,13 @@ __global__ void check(int n) {
     check_pair(a, b);
     check_pair(a, __uint_as_float(__float_as_uint(b) & 0xffff8000u));
     check_pair(a, 0.f);
+    // denominators 1 + x^2: any binade, all-ones and near-power fractions, and just above 1
+    const uint64_t ed = 1023 + (k2 >> 8) % ((i & 64) ? 1025 : 72);
+    const double dd = (i & 128) ? 1.0 + ldexp((double)(k >> 11), -53 - (int)(k2 % 60))
+                               : __longlong_as_double((long long)(ed << 52 | frac));
+    if (!same(rcp_ge1(dd), 1.0 / dd)) atomicAdd(&bad[5], 1ull);
+    const double dn = __longlong_as_double((long long)((ed << 52) + (long long)(k % 4096) - 2048));
+    if (dn >= 1.0 && !same(rcp_ge1(dn), 1.0 / dn)) atomicAdd(&bad[5], 1ull);
     if (dbl_of_int(1 + i % 2001) != (double)(1 + i % 2001)) atomicAdd(&bad[4], 1ull);
     const int m = (int)(k >> 34);   // below 2^30
     const ff c = ff_of_int(m), d = ff_of((double)m);
@@ -75,9 +82,9 @@ __global__ void check(int n) {
 }
 int main() {
   check<<<304, 256>>>(1 << 22);
-  unsigned long long h[5];
+  unsigned long long h[6];
   if (cudaMemcpyFromSymbol(h, bad, sizeof(h)) != cudaSuccess) return 1;
-  printf("%llu %llu %llu %llu %llu\n", h[0], h[1], h[2], h[3], h[4]);
+  printf("%llu %llu %llu %llu %llu %llu\n", h[0], h[1], h[2], h[3], h[4], h[5]);
   return 0;
 }
 """
@@ -90,4 +97,4 @@ def test_integer_conversions_match_fp64(tmp_path):
     subprocess.run([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-O2", "-std=c++17", "-I", CSRC, "-o",
                     str(exe), str(src)], check=True, capture_output=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
-    assert out == ["0"] * 5, dict(zip(("ff_of", "dbl_of", "ff_round53", "tab_segment", "integers"), out))
+    assert out == ["0"] * 6, dict(zip(("ff_of", "dbl_of", "ff_round53", "tab_segment", "integers", "rcp_ge1"), out))
