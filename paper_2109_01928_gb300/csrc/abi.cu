@@ -174,9 +174,11 @@ int debye_ctx::prep_spectra(const debye_spectra* sp, const Plan& pl, cudaStream_
 // Column-sum tables (DEBYE_PREC_MIXED_TABLE). Spectrum s gets nseg_s = ceil((hi - lo) /
 // TAB_W) segments from its lower bound; its nseg_s TAB_NC Chebyshev nodes are the poles
 // of ceil(nseg_s TAB_NC / TAB_NODE_N) pseudo-candidates of TAB_NODE_N poles, whose column
-// sums (with the derivative sums) the float-float column-sum pass computes; the
-// coefficients follow by a discrete cosine transform of the node values in FP64.
-int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, cudaStream_t st) {
+// sums (with_grad: and derivative sums) the float-float column-sum pass computes; the
+// coefficients follow by a discrete cosine transform of the node values in FP64. Without
+// with_grad the derivative functions are neither summed nor tabulated (1024 spectra, K
+// 50-1000: 496 us against 954).
+int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_grad, cudaStream_t st) {
   if (opt.precision != DEBYE_PREC_MIXED_TABLE || pl.S == 0) return DEBYE_OK;
   const int64_t S = pl.S;
   std::vector<double> lo(S), hi(S);
@@ -205,7 +207,7 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, cudaStream_
   if ((rc = named("tab.seg0", sizeof(int64_t) * S, &d_seg0)) || (rc = named("tab.nseg", sizeof(int32_t) * S, &d_nseg)) ||
       (rc = named("tab.qn0", sizeof(int32_t) * (S + 1), &d_qn0)) ||
       (rc = named("tab.theta", sizeof(double) * TAB_NODE_N * qn, &d_th)) ||
-      (rc = named("tab.G", sizeof(double) * 4 * TAB_NODE_N * qn, &d_G)) ||
+      (rc = named("tab.G", sizeof(double) * (with_grad ? 4 : 2) * TAB_NODE_N * qn, &d_G)) ||
       (rc = named("tab.x", sizeof(double) * TAB_NODE_N * qn, &d_x)) ||
       (rc = named("tab.coef", sizeof(float2) * TAB_NF * TAB_NC * segs, &d_coef)))
     return rc;
@@ -213,8 +215,10 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, cudaStream_
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_nseg, nseg.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_qn0, qn0.data(), sizeof(int32_t) * (S + 1), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return fail(DEBYE_ECUDA, "uploading the table plan: %s", cudaGetErrorString(e));
-  // node pass: TAB_NODE_N poles per pseudo-candidate, 16 pseudo-candidates x 8 lanes per block
-  constexpr int CBN = 16, KSN = 8;
+  // node pass: TAB_NODE_N poles per pseudo-candidate, 8 pseudo-candidates x 8 lanes per block
+  // (a box of 8 decades has 24 pseudo-candidates: with 16 per block, every second block of a
+  // spectrum was half empty: 1132 -> 954 us with the derivatives)
+  constexpr int CBN = 8, KSN = 8;
   Plan pn = pl;
   std::fill(pn.npol.begin(), pn.npol.end(), TAB_NODE_N);
   std::vector<int32_t> qb(qn0.begin(), qn0.end() - 1), qe(qn0.begin() + 1, qn0.end());
@@ -244,9 +248,9 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, cudaStream_
   if (prof_on) prof_begin(DEBYE_KERNEL_TABLE, 0.0, st, pe);
   launch_tab_nodes(S, (const int32_t*)d_qn0, (const int32_t*)d_nseg, sp->lo, (double*)d_th, sms, st);
   if (an.n_units > 0)
-    launch_pass(TAB_NODE_N, PH_SUMSG, an, std::max(1, std::min(an.n_units, sms * 16)), CBN * KSN, st);
+    launch_pass(TAB_NODE_N, with_grad ? PH_SUMSG : PH_SUMS, an, std::max(1, std::min(an.n_units, sms * 16)), CBN * KSN, st);
   launch_tab_coef(S, (const int32_t*)d_qn0, (const int32_t*)d_nseg, (const int64_t*)d_seg0, (const double*)d_G,
-                  (const double*)d_x, qn, (float2*)d_coef, sms, st);
+                  (const double*)d_x, qn, with_grad, (float2*)d_coef, sms, st);
   if (prof_on) prof_end(pe, st);
   launches += 3;
   tab.coef = (const float2*)d_coef;
@@ -472,7 +476,8 @@ struct EvalSetup {
 
 // Validate, plan and upload one evaluation; `layout` (cb > 0) replaces the layout rule.
 static int setup_eval(debye_handle h, const debye_spectra* sp, int32_t P, int32_t n_max, const double* theta,
-                      const double* cost, int32_t* n_failed, Layout layout, cudaStream_t st, EvalSetup& es) {
+                      const double* cost, bool with_grad, int32_t* n_failed, Layout layout, cudaStream_t st,
+                      EvalSetup& es) {
   if (P < 1) return h->fail(DEBYE_EINVAL, "P = %d < 1", P);
   if (n_max < 1 || n_max > NMAX) return h->fail(DEBYE_EINVAL, "n_max = %d outside 1..%d", n_max, NMAX);
   if (!sp) return h->fail(DEBYE_EINVAL, "spectra is NULL");
@@ -485,7 +490,7 @@ static int setup_eval(debye_handle h, const debye_spectra* sp, int32_t P, int32_
   if (es.empty) return DEBYE_OK;
   if (!theta || !cost) return h->fail(DEBYE_EINVAL, "theta or cost is NULL");
   if ((rc = h->prep_spectra(sp, pl, st))) return rc;
-  if ((rc = h->build_tables(sp, pl, st))) return rc;
+  if ((rc = h->build_tables(sp, pl, with_grad, st))) return rc;
   std::vector<int32_t> qb(pl.S), qe(pl.S);
   for (int64_t s = 0; s < pl.S; ++s) {
     qb[s] = (int32_t)(s * P);
@@ -537,7 +542,7 @@ static int eval_entry(debye_handle h, const debye_spectra* sp, int32_t P, int32_
   if (!h) return DEBYE_EINVAL;
   h->err.clear();
   EvalSetup es;
-  int rc = setup_eval(h, sp, P, n_max, theta, cost, n_failed, Layout{}, st, es);
+  int rc = setup_eval(h, sp, P, n_max, theta, cost, grad != nullptr, n_failed, Layout{}, st, es);
   return rc ? rc : run_setup(h, es, cost, weights, grad, st);
 }
 
@@ -753,7 +758,7 @@ int debye_autotune(debye_handle h, const debye_spectra* sp, int32_t P, int32_t n
     for (int round = -1; round < ROUNDS; ++round) {   // round -1: warm-up (workspaces, caches)
       for (int li = 0; li < n_set; ++li) {
         EvalSetup es;
-        int r = setup_eval(h, sp, Pe, n_max, th, c, nullptr, set[li], st, es);
+        int r = setup_eval(h, sp, Pe, n_max, th, c, gr != nullptr, nullptr, set[li], st, es);
         if (r) return r;
         if ((r = run_setup(h, es, c, nullptr, gr, st))) return r;   // untimed: first launch of each kernel
         // captured and replayed on the handle's own stream (the caller's may be the legacy

@@ -86,7 +86,8 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
   const int64_t Q = pl.S * (int64_t)P;
   if (Q > ((int64_t)1 << 31) - 1) return h->fail(DEBYE_EINVAL, "S*P exceeds 2^31-1");
   if ((rc = h->prep_spectra(sp, pl, st))) return rc;
-  if ((rc = h->build_tables(sp, pl, st))) return rc;   // once per fit: the samples do not change
+  // once per fit: the samples do not change; only the polish needs gradients
+  if ((rc = h->build_tables(sp, pl, std::min(se->polish_topk, se->P) > 0, st))) return rc;
   int cb, ks;
   choose_layout(P, Q, h->sms, h->forced(), h->tuned, &cb, &ks);
   const bool mixed = h->mixed();

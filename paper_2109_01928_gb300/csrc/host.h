@@ -109,7 +109,7 @@ struct debye_ctx {
   bool mixed() const { return opt.precision == DEBYE_PREC_MIXED || opt.precision == DEBYE_PREC_MIXED_TABLE; }
   // DEBYE_PREC_MIXED_TABLE: build every spectrum's column-sum tables (after
   // prep_spectra) and point `tab` at them; a no-op for the other precisions.
-  int build_tables(const debye_spectra* sp, const debyefit::Plan& pl, cudaStream_t st);
+  int build_tables(const debye_spectra* sp, const debyefit::Plan& pl, bool with_grad, cudaStream_t st);
   int named(const char* name, size_t bytes, void** out);
 
   void free_buf(debyefit::Buf& b) {

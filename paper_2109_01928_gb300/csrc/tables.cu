@@ -73,11 +73,11 @@ __global__ void k_tab_nodes(int64_t S, const int32_t* qn0, const int32_t* nseg, 
 // the column-sum pass wrote S, h, dS, dh at G[(r TAB_NODE_N + i) Qn + q], r = 0..3, and
 // tau at X[i Qn + q].
 __global__ void k_tab_coef(int64_t S, const int32_t* qn0, const int32_t* nseg, const int64_t* seg0,
-                           ChebConst cc, const double* G, const double* X, int64_t Qn, float2* coef) {
+                           ChebConst cc, const double* G, const double* X, int64_t Qn, int nf, float2* coef) {
   for (int64_t s = blockIdx.x; s < S; s += gridDim.x) {
-    const int items = nseg[s] * TAB_NF;
+    const int items = nseg[s] * nf;   // nf: the functions tabulated, the first 3 or all
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
-      const int g = it / TAB_NF, f = it % TAB_NF;
+      const int g = it / nf, f = it % nf;
       double v[TAB_NC];
 #pragma unroll
       for (int m = 0; m < TAB_NC; ++m) {
@@ -237,9 +237,9 @@ void launch_tab_nodes(int64_t S, const int32_t* qn0, const int32_t* nseg, const 
 }
 
 void launch_tab_coef(int64_t S, const int32_t* qn0, const int32_t* nseg, const int64_t* seg0, const double* G,
-                     const double* X, int64_t Qn, float2* coef, int sms, cudaStream_t st) {
+                     const double* X, int64_t Qn, bool with_grad, float2* coef, int sms, cudaStream_t st) {
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(S, (int64_t)sms * 32));
-  k_tab_coef<<<grid, 128, 0, st>>>(S, qn0, nseg, seg0, cheb_const(), G, X, Qn, coef);
+  k_tab_coef<<<grid, 128, 0, st>>>(S, qn0, nseg, seg0, cheb_const(), G, X, Qn, with_grad ? TAB_NF : 3, coef);
 }
 
 void launch_tab_eval(const EvalArgs& a, bool grad, int sms, cudaStream_t st) {
