@@ -348,7 +348,7 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
   // units) for every non-empty bucket below b_hi; kind >= 0 times the whole fork-join.
   // The buckets are launched from the fewest poles up: measured on a whole mixed_1024
   // fit step (graphs on), this order is 12-15 % faster than launching the most poles
-  // first.
+  // first (and for the table precision's solves alone: fits 71.8 ms against 76.2).
   auto fork_buckets = [&](int kind, double flops, int b_hi, auto body) -> int {
     int first = -1, n_nonempty = 0;
     for (int b = 0; b < b_hi; ++b)
