@@ -432,9 +432,19 @@ __global__ void __launch_bounds__(32) k_solve_rows(EvalArgs a, int slices, doubl
       for (int i = 1; i < N; ++i) {
         const ff ti = tau_of(i), pi = ff_prod(ti, M.get(pk(i + 1, 0)));
 #pragma unroll
-        for (int j = 0; j < N - 1; ++j) {
-          if (j >= i) break;
-          M.put(pk(i + 1, j + 1), ff_quot(ff_sum(pi, pr[j]), ff_sum(ti, tau[j])));
+        for (int j0 = 0; j0 < N - 1; j0 += 4) {   // four independent quotients at a time
+          if (j0 >= i) break;
+          ff g[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const int j = j0 + t;
+            if (j < N - 1) g[t] = ff_quot(ff_sum(pi, pr[j]), ff_sum(ti, tau[j]));
+          }
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const int j = j0 + t;
+            if (j < N - 1 && j < i) M.put(pk(i + 1, j + 1), g[t]);
+          }
         }
       }
     }
