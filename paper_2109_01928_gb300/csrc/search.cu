@@ -50,32 +50,55 @@ __device__ __forceinline__ double u53_double(uint64_t u) {
   return __longlong_as_double((long long)(((uint64_t)(e + 1023) << 52) | mant));
 }
 
-__global__ void k_pso_move(SwarmArgs a) {
-  const int64_t Q = (int64_t)a.S * a.P;
+// fmin(fmax(v, lo), hi) by integer comparisons (an FP64 one holds the FP64 pipe as long as
+// an FP64 addition); with a NaN or infinite operand, the FP64 form.
+__device__ __forceinline__ long long ordered_bits(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ (long long)((unsigned long long)(b >> 63) >> 1);
+}
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ double clamp_to(double v, double lo, double hi) {
+  if (!(finite_bits(v) && finite_bits(lo) && finite_bits(hi))) return fmin(fmax(v, lo), hi);
+  if (ordered_bits(v) < ordered_bits(lo)) v = lo;
+  return ordered_bits(v) > ordered_bits(hi) ? hi : v;
+}
+
+// One thread per coordinate of a spectrum's swarm: rows are read and written contiguously
+// (a thread per particle strode through its row, re-reading every sector up to 4 times),
+// and the keys' prefixes, the same for a whole spectrum, are formed once per block. What is
+// left is the FP64 pipe: 10 operations per coordinate, 64 cycles per warp each.
+constexpr int MOVE_BLOCK = 256;
+__global__ void __launch_bounds__(MOVE_BLOCK) k_pso_move(SwarmArgs a, int chunks) {
+  __shared__ uint64_t prefix[2];
   const int gen = *a.gen;
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < Q;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t s = q / a.P, p = q % a.P;
+  const int rows = (a.P + chunks - 1) / chunks;   // particles of a block's turn
+  // phi r = phi (u 2^-53) = (phi 2^-53) u: the scaling by 2^-53 is exact, so both round
+  // the same exact product once and the update stays bit-identical to phi * r (for any
+  // |phi| >= 2^-969, where phi 2^-53 is still a normal number)
+  const double cp = __dmul_rn(a.phi_p, 0x1p-53), cg = __dmul_rn(a.phi_g, 0x1p-53);
+  for (int64_t w = blockIdx.x; w < a.S * chunks; w += gridDim.x) {
+    const int64_t s = w / chunks;
+    const int p0 = (int)(w % chunks) * rows, p1 = min(a.P, p0 + rows);
+    if (threadIdx.x < 2)
+      prefix[threadIdx.x] = rng_prefix(a.seed, threadIdx.x ? TAG_R2 : TAG_R1, key_id(a, s), (uint64_t)gen);
+    __syncthreads();
     const int N = a.n_poles[s];
     const double lo = a.lo[s], hi = a.hi[s];
-    const int64_t gq = s * a.P + a.gbest[s];
-    const uint64_t p1 = rng_prefix(a.seed, TAG_R1, key_id(a, s), (uint64_t)gen);
-    const uint64_t p2 = rng_prefix(a.seed, TAG_R2, key_id(a, s), (uint64_t)gen);
-    // phi r = phi (u 2^-53) = (phi 2^-53) u: the scaling by 2^-53 is exact, so both round
-    // the same exact product once and the update stays bit-identical to phi * r (for any
-    // |phi| >= 2^-969, where phi 2^-53 is still a normal number)
-    const double cp = __dmul_rn(a.phi_p, 0x1p-53), cg = __dmul_rn(a.phi_g, 0x1p-53);
-    for (int d = 0; d < N; ++d) {
-      const double x = a.x[q * a.nmax + d], v = a.v[q * a.nmax + d];
-      const double pb = a.pbx[q * a.nmax + d], gb = a.pbx[gq * a.nmax + d];
-      const double u1 = u53_double(rng_key(p1, p, d) >> 11), u2 = u53_double(rng_key(p2, p, d) >> 11);
+    const int64_t row0 = s * a.P;
+    const double* best = a.pbx + (row0 + a.gbest[s]) * a.nmax;
+    for (int e = p0 * N + (int)threadIdx.x; e < p1 * N; e += MOVE_BLOCK) {
+      const int p = e / N, d = e - p * N;
+      const int64_t at = (row0 + p) * a.nmax + d;
+      const double x = a.x[at], v = a.v[at], pb = a.pbx[at], gb = best[d];
+      const double u1 = u53_double(rng_key(prefix[0], p, d) >> 11), u2 = u53_double(rng_key(prefix[1], p, d) >> 11);
       const double t1 = __dmul_rn(a.omega, v);
       const double t2 = __dmul_rn(__dmul_rn(cp, u1), __dsub_rn(pb, x));
       const double t3 = __dmul_rn(__dmul_rn(cg, u2), __dsub_rn(gb, x));
       const double vn = __dadd_rn(__dadd_rn(t1, t2), t3);
-      a.v[q * a.nmax + d] = vn;
-      a.x[q * a.nmax + d] = fmin(fmax(__dadd_rn(x, vn), lo), hi);
+      a.v[at] = vn;
+      a.x[at] = clamp_to(__dadd_rn(x, vn), lo, hi);
     }
+    __syncthreads();   // the prefixes are read before the next turn's are written
   }
 }
 
@@ -652,7 +675,10 @@ void launch_pso_init(const SwarmArgs& a, int sms, cudaStream_t st) {
   k_pso_init<<<g1d((int64_t)a.S * a.P, sms), 256, 0, st>>>(a);
 }
 void launch_pso_move(const SwarmArgs& a, int sms, cudaStream_t st) {
-  k_pso_move<<<g1d((int64_t)a.S * a.P, sms), 256, 0, st>>>(a);
+  // enough turns to fill the GPU, each of at least 16 particles
+  const int64_t want = (int64_t)sms * 8;
+  const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>((want + a.S - 1) / a.S, (a.P + 15) / 16));
+  k_pso_move<<<(int)std::min<int64_t>(a.S * chunks, (int64_t)sms * 32), MOVE_BLOCK, 0, st>>>(a, chunks);
 }
 void launch_de_trial(const SwarmArgs& a, int sms, cudaStream_t st) {
   k_de_trial<<<g1d((int64_t)a.S * a.P, sms), 256, 0, st>>>(a);
