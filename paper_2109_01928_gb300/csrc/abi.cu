@@ -257,6 +257,7 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
   tab.seg0 = (const int64_t*)d_seg0;
   tab.nseg = (const int32_t*)d_nseg;
   tab.lo = sp->lo;
+  tab_max_seg = *std::max_element(nseg.begin(), nseg.end());
   return check_launch("column-sum tables");
 }
 
@@ -431,7 +432,7 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
     if (opt.precision == DEBYE_PREC_MIXED_TABLE) {
       // the sums of every candidate from the tables (one launch), then the solves
       a.tab = tab;
-      timed(DEBYE_KERNEL_TABLE_EVAL, [&] { launch_tab_eval(a, grad != nullptr, sms, st); });
+      timed(DEBYE_KERNEL_TABLE_EVAL, [&] { launch_tab_eval(a, grad != nullptr, tab_max_seg, sms, st); });
       rc = fork_buckets(prof_on ? DEBYE_KERNEL_SOLVE : -1, 0.0, nb_n, solve_bucket);
     } else if (!prof_on) {
       rc = fork_buckets(-1, 0.0, N_BUCKETS, [&](int b, const EvalArgs& ab, cudaStream_t bs) {

@@ -71,6 +71,7 @@ struct debye_ctx {
   debyefit::Buf ws_kq, ws_h0, ws_units;
   debyefit::Buf ws_tab_units;    // units of the column-sum tables' node pass
   debyefit::TabView tab{};       // column-sum tables of the current call (DEBYE_PREC_MIXED_TABLE)
+  int tab_max_seg = 0;           // the most segments of a spectrum
   debyefit::ScratchBufs sb_eval, sb_polish, sb_polish_acc, sb_final;
   std::map<std::string, debyefit::Buf> named_bufs;  // swarm / polish / result state
 

@@ -99,7 +99,7 @@ void launch_tab_nodes(int64_t S, const int32_t* qn0, const int32_t* nseg, const 
                       int sms, cudaStream_t st);
 void launch_tab_coef(int64_t S, const int32_t* qn0, const int32_t* nseg, const int64_t* seg0, const double* G,
                      const double* X, int64_t Qn, bool with_grad, float2* coef, int sms, cudaStream_t st);
-void launch_tab_eval(const EvalArgs& a, bool grad, int sms, cudaStream_t st);
+void launch_tab_eval(const EvalArgs& a, bool grad, int max_seg, int sms, cudaStream_t st);
 // One block running the column-sum pass's bounded staging wait with nothing to wait
 // for (waitcheck.cu): it records DEBYE_ETIMEOUT after the wait's clock budget;
 // waited_ok (device, or nullptr) receives 0.

@@ -110,16 +110,15 @@ __global__ void k_tab_coef(int64_t S, const int32_t* qn0, const int32_t* nseg, c
 }
 
 // f(x) = sum_k a_k x^k for x in [-1, 1] by Horner's rule in float-float. The
-// coefficients are read two at a time (16-byte loads: every function's TAB_NC
-// coefficients start on a multiple of TAB_NC * 8 = 96 bytes from the allocation),
-// halving the load instructions, which bound this kernel on the L1 pipe.
+// coefficients (hi, lo) are read two at a time (16-byte loads: every function's TAB_NC
+// coefficients start on a multiple of TAB_NC * 8 = 96 bytes).
 static_assert(TAB_NC % 2 == 0 && (TAB_NC * sizeof(float2)) % 16 == 0, "paired coefficient loads");
-__device__ __forceinline__ ff poly_ff(const float2* __restrict__ a, ff x) {
-  const float4* a4 = reinterpret_cast<const float4*>(a);
-  float4 c[TAB_NC / 2];
+constexpr int TAB_F4 = TAB_NC / 2;   // float4 of one function
+__device__ __forceinline__ ff poly_ff(const float4* a4, ff x) {
+  float4 c[TAB_F4];
 #pragma unroll
-  for (int i = 0; i < TAB_NC / 2; ++i) c[i] = __ldg(a4 + i);
-  ff acc{c[TAB_NC / 2 - 1].z, c[TAB_NC / 2 - 1].w};
+  for (int i = 0; i < TAB_F4; ++i) c[i] = a4[i];
+  ff acc{c[TAB_F4 - 1].z, c[TAB_F4 - 1].w};
 #pragma unroll
   for (int k = TAB_NC - 2; k >= 0; --k) {
     const float4 q = c[k / 2];
@@ -183,9 +182,17 @@ __device__ __forceinline__ double dbl_of_int(uint32_t m) {
 // 2N + i, 3N + i, in float-float) for the column-sum solves. One thread per (candidate,
 // pole). With the position and the results converted by integer operations, 3 FP64
 // operations per pole are left of 20, whose pipe bound the kernel: 88 -> 67 us for 1024
-// spectra x 256 candidates, N 2-12.
+// spectra x 256 candidates, N 2-12. After that the gathers did: a warp's poles lie in some
+// 25 different segments, each a line of its own to the L1. A unit with at least two poles
+// per segment of its spectrum copies the spectrum's functions to shared memory first, at an
+// odd number of 16-byte words per segment, which spreads the segments over the banks:
+// 67 -> 56 us. smem_seg: segments the launch has shared memory for.
 template <bool GRAD>
-__global__ void __launch_bounds__(128) k_tab_eval(EvalArgs a) {
+__global__ void __launch_bounds__(128) k_tab_eval(EvalArgs a, int smem_seg) {
+  constexpr int NF = GRAD ? TAB_NF : 3;           // functions read
+  constexpr int GS = TAB_NF * TAB_F4, SS = NF * TAB_F4 + 1;   // float4 per segment: in memory, staged
+  static_assert(SS % 2 == 1, "segments spread over the banks");
+  extern __shared__ float4 tab_smem[];
   const int64_t Q = a.sc.Q;
   double* G = a.sc.G;
   for (int ui = blockIdx.x; ui < a.n_units; ui += gridDim.x) {
@@ -193,7 +200,16 @@ __global__ void __launch_bounds__(128) k_tab_eval(EvalArgs a) {
     const int nc = u.q1 - u.q0, N = u.N;
     const double l = a.tab.lo[u.s];
     const int ns = a.tab.nseg[u.s];
-    const float2* cs = a.tab.coef + a.tab.seg0[u.s] * (TAB_NF * TAB_NC);
+    const float4* cs = reinterpret_cast<const float4*>(a.tab.coef) + a.tab.seg0[u.s] * GS;
+    const bool staged = ns <= smem_seg && nc * N >= 2 * ns && !a.active;
+    if (staged) {
+      __syncthreads();   // the previous unit's functions are read
+      for (int e = threadIdx.x; e < ns * (SS - 1); e += blockDim.x) {
+        const int g = e / (SS - 1), c = e - g * (SS - 1);
+        tab_smem[g * SS + c] = __ldg(cs + (int64_t)g * GS + c);
+      }
+      __syncthreads();
+    }
     for (int p = threadIdx.x; p < nc * N; p += blockDim.x) {
       const int j = p / nc, q = u.q0 + p % nc;
       if (a.active && !a.active[q]) continue;
@@ -201,17 +217,20 @@ __global__ void __launch_bounds__(128) k_tab_eval(EvalArgs a) {
       const double d = th - l;
       const int g = tab_segment(d * TAB_INV_W, ns);
       ff tau, v[4];
+      auto eval = [&](const float4* c, ff x) {
+        v[0] = ff_round53(poly_ff(c, x));
+        v[1] = ff_round53(poly_ff(c + TAB_F4, x));
+        tau = ff_round53(poly_ff(c + 2 * TAB_F4, x));
+        if (GRAD) {
+          v[2] = ff_round53(poly_ff(c + 3 * TAB_F4, x));
+          v[3] = ff_round53(poly_ff(c + 4 * TAB_F4, x));
+        }
+      };
       if (g >= 0) {
         // x = 2 (uu - g) - 1 in [-1, 1]
         const ff x = ff_of(fma(d, 2.0 * TAB_INV_W, -dbl_of_int(2 * g + 1)));
-        const float2* c = cs + (int64_t)g * (TAB_NF * TAB_NC);
-        v[0] = ff_round53(poly_ff(c, x));
-        v[1] = ff_round53(poly_ff(c + TAB_NC, x));
-        tau = ff_round53(poly_ff(c + 2 * TAB_NC, x));
-        if (GRAD) {
-          v[2] = ff_round53(poly_ff(c + 3 * TAB_NC, x));
-          v[3] = ff_round53(poly_ff(c + 4 * TAB_NC, x));
-        }
+        if (staged) eval(tab_smem + g * SS, x);
+        else eval(cs + (int64_t)g * GS, x);
       } else {
         double s[4];
         const double t = exp10(th);
@@ -242,10 +261,14 @@ void launch_tab_coef(int64_t S, const int32_t* qn0, const int32_t* nseg, const i
   k_tab_coef<<<grid, 128, 0, st>>>(S, qn0, nseg, seg0, cheb_const(), G, X, Qn, with_grad ? TAB_NF : 3, coef);
 }
 
-void launch_tab_eval(const EvalArgs& a, bool grad, int sms, cudaStream_t st) {
+// max_seg: the most segments of a spectrum. Shared memory for up to 64 segments (box of 12.8
+// decades, 19.5 KB, 31.7 KB with the derivatives); larger tables are read where they are.
+void launch_tab_eval(const EvalArgs& a, bool grad, int max_seg, int sms, cudaStream_t st) {
   const int grid = std::max(1, std::min(a.n_units, sms * 16));
-  if (grad) k_tab_eval<true><<<grid, 128, 0, st>>>(a);
-  else k_tab_eval<false><<<grid, 128, 0, st>>>(a);
+  const int seg = max_seg <= 64 ? max_seg : 0;
+  const size_t smem = (size_t)seg * ((grad ? TAB_NF : 3) * TAB_F4 + 1) * sizeof(float4);
+  if (grad) k_tab_eval<true><<<grid, 128, smem, st>>>(a, seg);
+  else k_tab_eval<false><<<grid, 128, smem, st>>>(a, seg);
 }
 
 }  // namespace debyefit
