@@ -272,12 +272,16 @@ __device__ __forceinline__ ff ff_of_int(int v) {
   const float h = __int2float_rn(v);
   return ff{h, __int2float_rn(v - (int)h)};
 }
+// The plain forms behind the integer ones are calls, so that they are branched around: as
+// predicated instructions they would hold the FP64 pipe even when not taken.
+static __device__ __noinline__ double dbl_of_plain(float a) { return (double)a; }
 // The FP64 value of an FP32 one.
 __device__ __forceinline__ double dbl_of(float a) {
   const uint32_t b = __float_as_uint(a), m = b & 0x7fffffffu;
   if (m - 0x00800000u < 0x7f000000u)   // normal
     return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + (896u << 20))), (int)(b << 29));
-  return m == 0 ? __hiloint2double((int)b, 0) : (double)a;
+  if (m == 0) return __hiloint2double((int)b, 0);
+  return dbl_of_plain(a);
 }
 // ff_of((double)a.h + (double)a.l) of a normalised a: the low part rounded to the last bit
 // of the sum's FP64 value, by adding and removing a power of two whose last bit that is.

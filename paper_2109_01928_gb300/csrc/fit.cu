@@ -20,6 +20,10 @@ namespace {
 
 // Line search of the polish: the full step is evaluated first (with its gradient);
 // a line that rejects it evaluates POLISH_R further step lengths per backtracking round.
+// Where so few lines are polished that all their step lengths together leave the GPU
+// unfilled (one warp per candidate's solve, see solve_sums_by_warp), one round evaluates
+// every step length: the rounds after the first, idle as a rule, cost their launches only
+// (one spectrum, 8 lines: 7 launches fewer per iteration). A round is at most 32 trials.
 constexpr int POLISH_R = 8;
 
 struct GraphGuard {
@@ -142,6 +146,8 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
   sa.gbest = (int32_t*)p;
   if ((rc = h->named("swarm.gen", sizeof(int), &p))) return rc;
   sa.gen = (int*)p;
+  if ((rc = h->named("swarm.gens", sizeof(int) * pl.S, &p))) return rc;
+  sa.gens = (int*)p;
   if (anneal) {
     if ((rc = h->named("anneal.cx", qn, &p))) return rc;
     sa.cx = (double*)p;
@@ -154,6 +160,7 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
   sa.evals = se->evals;
   if (se->evals && reset_evals) cudaMemsetAsync(se->evals, 0, sizeof(double), st);
   cudaMemsetAsync(sa.gen, 0, sizeof(int), st);
+  cudaMemsetAsync(sa.gens, 0, sizeof(int) * pl.S, st);
 
   ea.units = (const Unit*)h->ws_units.p;
   ea.theta = sa.x;
@@ -175,12 +182,17 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
   // generation 0: initial positions (the same for both methods), evaluation, bests
   launch_pso_init(sa, h->sms, st); ++h->launches;
   if ((rc = h->run_eval(ea, g, mixed, steps, cost, nullptr, nullptr, h->sb_eval.g1, cb, st))) return rc;
-  launch_pso_best(sa, cost, h->sms, st); ++h->launches;
-  if (anneal) {
-    launch_da_start(sa, h->sms, st);
-    ++h->launches;
+  // the swarm: bests and the next generation's move in one kernel where a block takes a
+  // whole population
+  const bool swarm_step = !evolve && !anneal && P <= PSO_STEP_MAX_P;
+  if (!swarm_step) {
+    launch_pso_best(sa, cost, h->sms, st); ++h->launches;
+    if (anneal) {
+      launch_da_start(sa, h->sms, st);
+      ++h->launches;
+    }
+    launch_gen_advance(sa.gen, st); ++h->launches;
   }
-  launch_gen_advance(sa.gen, st); ++h->launches;
   if ((rc = h->check_launch("swarm start"))) return rc;
   if (anneal) {
     // one outer iteration: 2 nmax moves (moves beyond 2 N_s are masked for spectrum s),
@@ -198,6 +210,14 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
       launch_gen_advance(sa.gen, st); ++h->launches;
       return h->check_launch("annealing iteration");
     });
+  } else if (swarm_step) {
+    rc = repeat(h, se->iters, st, [&]() -> int {
+      launch_pso_step(sa, cost, true, h->sms, st); ++h->launches;
+      int r = h->run_eval(ea, g, mixed, steps, cost, nullptr, nullptr, h->sb_eval.g1, cb, st);
+      return r ? r : h->check_launch("generation");
+    });
+    if (rc) return rc;
+    launch_pso_step(sa, cost, false, h->sms, st); ++h->launches;
   } else rc = repeat(h, se->iters, st, [&]() -> int {
     if (evolve) launch_de_trial(sa, h->sms, st);
     else launch_pso_move(sa, h->sms, st);
@@ -217,6 +237,10 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
   if (T > 0) {
     pa.L = pl.S * (int64_t)T;
     pa.R = POLISH_R;
+    // (the failure counter counts evaluated candidates, so it keeps the rounds)
+    if (h->opt.lbfgs_max_trials > 1 + POLISH_R && h->opt.lbfgs_max_trials <= 33 && !se->n_failed &&
+        solve_sums_by_warp(pa.L * (h->opt.lbfgs_max_trials - 1), 0, h->sms))
+      pa.R = h->opt.lbfgs_max_trials - 1;
     pa.nmax = nmax;
     pa.m = h->opt.lbfgs_m;
     pa.max_trials = h->opt.lbfgs_max_trials;
@@ -236,11 +260,15 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
     pa.hs = (double*)p;
     if ((rc = h->named("pol.hy", ln * pa.m, &p))) return rc;
     pa.hy = (double*)p;
-    if ((rc = h->named("pol.int", sizeof(int32_t) * 4 * L, &p))) return rc;
+    if ((rc = h->named("pol.rho", sizeof(double) * L * (pa.m + 1), &p))) return rc;
+    pa.rho = (double*)p;
+    pa.gamma = pa.rho + L * pa.m;
+    if ((rc = h->named("pol.int", sizeof(int32_t) * 5 * L, &p))) return rc;
     pa.hcount = (int32_t*)p;
     pa.t0 = pa.hcount + L;
     pa.done = pa.hcount + 2 * L;
     pa.acc = pa.hcount + 3 * L;
+    pa.head = pa.hcount + 4 * L;
     if ((rc = h->named("pol.tth", sizeof(double) * QT * nmax, &p))) return rc;
     pa.tth = (double*)p;
     if ((rc = h->named("pol.tcost", sizeof(double) * QT, &p))) return rc;
@@ -264,10 +292,11 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
       ab[s] = (int32_t)(s * T);
       ae[s] = (int32_t)((s + 1) * T);
     }
-    // trial steps: one work unit per line (its R step lengths), so that a unit whose line
-    // has stopped searching exits at once and an active one has no idle candidates
+    // trial steps: POLISH_R candidates per work unit (a line's step lengths of a round), so
+    // that a unit whose line has stopped searching exits at once and an active one has no
+    // idle candidates
     int cba, ksa;
-    const int cbp = pa.R, ksp = MAX_BLOCK / pa.R;
+    const int cbp = POLISH_R, ksp = MAX_BLOCK / POLISH_R;
     if (h->tuned_polish.cb > 0) {   // debye_autotune's choice for this shape
       cba = h->tuned_polish.cb;
       ksa = h->tuned_polish.ks;
@@ -306,7 +335,8 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
     if ((rc = h->check_launch("polish start"))) return rc;
     const int rounds = (pa.max_trials - 1 + pa.R - 1) / pa.R;
     rc = repeat(h, se->polish_iters, st, [&]() -> int {
-      launch_polish_dir(pa, sp->n_poles, sp->lo, sp->hi, h->sms, st); ++h->launches;
+      // the previous iteration's L-BFGS update and this one's direction
+      launch_polish_step(pa, sp->n_poles, sp->lo, sp->hi, h->sms, st); ++h->launches;
       // the full step of every line, with its gradient (most lines accept it)
       int e = h->run_eval(eg, ga, mixed, h->eval_steps(true), pa.acost, nullptr, pa.agrad, h->sb_polish_acc.g1,
                           cba, st);
@@ -318,14 +348,14 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
         if (e) return e;
         launch_polish_accept(pa, sp->n_poles, sp->lo, sp->hi, sp->offsets, h->sms, st); ++h->launches;
       }
-      // cost and gradient at the points accepted by backtracking, then the L-BFGS update
+      // cost and gradient at the points accepted by backtracking
       e = h->run_eval(eg, ga, mixed, h->eval_steps(true), pa.acost, nullptr, pa.agrad, h->sb_polish_acc.g1, cba,
                       st);
       if (e) return e;
-      launch_polish_take(pa, sp->n_poles, h->sms, st); ++h->launches;
       return h->check_launch("polish iteration");
     });
     if (rc) return rc;
+    launch_polish_take(pa, sp->n_poles, h->sms, st); ++h->launches;
   }
 
   // ---- final FP64 re-solve at lam_final, sorted result

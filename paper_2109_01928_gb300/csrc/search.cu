@@ -6,6 +6,7 @@
 // __d*_rn operations (no FMA contraction) so that positions are bit-identical
 // to an FP64 implementation evaluating
 //   v = (omega v + (phi_p r1) (p - x)) + (phi_g r2) (g - x),  x = clip(x + v, lo, hi).
+#include <climits>
 #include <cmath>
 
 #include "dmath.cuh"
@@ -57,25 +58,71 @@ __device__ __forceinline__ long long ordered_bits(double v) {
   return b ^ (long long)((unsigned long long)(b >> 63) >> 1);
 }
 __device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+// (calls, so that they are branched around: predicated, they would hold the pipe all the same)
+static __device__ __noinline__ double clamp_plain(double v, double lo, double hi) { return fmin(fmax(v, lo), hi); }
+static __device__ __noinline__ double mul_plain(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double clamp_to(double v, double lo, double hi) {
-  if (!(finite_bits(v) && finite_bits(lo) && finite_bits(hi))) return fmin(fmax(v, lo), hi);
+  if (!(finite_bits(v) && finite_bits(lo) && finite_bits(hi))) return clamp_plain(v, lo, hi);
   if (ordered_bits(v) < ordered_bits(lo)) v = lo;
   return ordered_bits(v) > ordered_bits(hi) ? hi : v;
+}
+
+// The swarm update's coefficients. phi r = phi (u 2^-53) = (phi 2^-53) u: the scaling by
+// 2^-53 is exact, so both round the same exact product once and the update stays
+// bit-identical to phi * r (for any |phi| >= 2^-969, where phi 2^-53 is still a normal
+// number). A positive power of two (the defaults are 0.5) multiplies by adding to the
+// exponent, off the FP64 pipe.
+struct MoveCoef {
+  double omega, cp, cg;
+  int eo, ep, eg;   // exponents of omega, cp, cg if powers of two, else INT_MIN
+  static __device__ __forceinline__ int pow2(double v) {
+    const int hi = __double2hiint(v);
+    return (hi & 0xfffff) == 0 && __double2loint(v) == 0 && hi > 0x00100000 && hi < 0x7fe00000 ? (hi >> 20) - 1023
+                                                                                           : INT_MIN;
+  }
+  static __device__ __forceinline__ MoveCoef of(const SwarmArgs& a) {
+    MoveCoef c;
+    c.omega = a.omega;
+    c.cp = __dmul_rn(a.phi_p, 0x1p-53);
+    c.cg = __dmul_rn(a.phi_g, 0x1p-53);
+    c.eo = pow2(c.omega);
+    c.ep = pow2(c.cp);
+    c.eg = pow2(c.cg);
+    return c;
+  }
+  // c v, c = 2^e where e != INT_MIN: exact unless the product leaves the normal range
+  static __device__ __forceinline__ double mul(double c, int e, double v) {
+    const int hi = __double2hiint(v), ev = (hi >> 20) & 0x7ff;
+    if (e != INT_MIN && ev != 0 && ev != 0x7ff && ev + e > 0 && ev + e < 0x7ff)
+      return __hiloint2double(hi + (e << 20), __double2loint(v));
+    return mul_plain(c, v);
+  }
+};
+
+// One coordinate: new velocity (returned) and position of x.
+__device__ __forceinline__ double move_one(const MoveCoef& c, uint64_t key1, uint64_t key2, double& x, double v,
+                                           double pb, double gb, double lo, double hi) {
+  const double u1 = u53_double(key1 >> 11), u2 = u53_double(key2 >> 11);
+  const double t1 = MoveCoef::mul(c.omega, c.eo, v);
+  const double t2 = __dmul_rn(MoveCoef::mul(c.cp, c.ep, u1), __dsub_rn(pb, x));
+  const double t3 = __dmul_rn(MoveCoef::mul(c.cg, c.eg, u2), __dsub_rn(gb, x));
+  const double vn = __dadd_rn(__dadd_rn(t1, t2), t3);
+  x = clamp_to(__dadd_rn(x, vn), lo, hi);
+  return vn;
 }
 
 // One thread per coordinate of a spectrum's swarm: rows are read and written contiguously
 // (a thread per particle strode through its row, re-reading every sector up to 4 times),
 // and the keys' prefixes, the same for a whole spectrum, are formed once per block. What is
-// left is the FP64 pipe: 10 operations per coordinate, 64 cycles per warp each.
+// left is the FP64 pipe: 7 operations per coordinate (10 with coefficients that are no
+// powers of two), 64 cycles per warp each. 1024 spectra x 256 particles, N 2-12: 83 -> 57
+// us. It serves populations beyond PSO_STEP_MAX_P; smaller ones take k_pso_step.
 constexpr int MOVE_BLOCK = 256;
 __global__ void __launch_bounds__(MOVE_BLOCK) k_pso_move(SwarmArgs a, int chunks) {
   __shared__ uint64_t prefix[2];
   const int gen = *a.gen;
   const int rows = (a.P + chunks - 1) / chunks;   // particles of a block's turn
-  // phi r = phi (u 2^-53) = (phi 2^-53) u: the scaling by 2^-53 is exact, so both round
-  // the same exact product once and the update stays bit-identical to phi * r (for any
-  // |phi| >= 2^-969, where phi 2^-53 is still a normal number)
-  const double cp = __dmul_rn(a.phi_p, 0x1p-53), cg = __dmul_rn(a.phi_g, 0x1p-53);
+  const MoveCoef co = MoveCoef::of(a);
   for (int64_t w = blockIdx.x; w < a.S * chunks; w += gridDim.x) {
     const int64_t s = w / chunks;
     const int p0 = (int)(w % chunks) * rows, p1 = min(a.P, p0 + rows);
@@ -89,14 +136,9 @@ __global__ void __launch_bounds__(MOVE_BLOCK) k_pso_move(SwarmArgs a, int chunks
     for (int e = p0 * N + (int)threadIdx.x; e < p1 * N; e += MOVE_BLOCK) {
       const int p = e / N, d = e - p * N;
       const int64_t at = (row0 + p) * a.nmax + d;
-      const double x = a.x[at], v = a.v[at], pb = a.pbx[at], gb = best[d];
-      const double u1 = u53_double(rng_key(prefix[0], p, d) >> 11), u2 = u53_double(rng_key(prefix[1], p, d) >> 11);
-      const double t1 = __dmul_rn(a.omega, v);
-      const double t2 = __dmul_rn(__dmul_rn(cp, u1), __dsub_rn(pb, x));
-      const double t3 = __dmul_rn(__dmul_rn(cg, u2), __dsub_rn(gb, x));
-      const double vn = __dadd_rn(__dadd_rn(t1, t2), t3);
-      a.v[at] = vn;
-      a.x[at] = clamp_to(__dadd_rn(x, vn), lo, hi);
+      double x = a.x[at];
+      a.v[at] = move_one(co, rng_key(prefix[0], p, d), rng_key(prefix[1], p, d), x, a.v[at], a.pbx[at], best[d], lo, hi);
+      a.x[at] = x;
     }
     __syncthreads();   // the prefixes are read before the next turn's are written
   }
@@ -283,6 +325,17 @@ __device__ __forceinline__ void argmin_merge(double& c, int& i, double c2, int i
     i = i2;
   }
 }
+// The same on a cost's ordered bits (no NaN; a negative zero as a positive one).
+__device__ __forceinline__ long long cost_key(double c) {
+  const long long b = __double_as_longlong(c);
+  return b == (long long)0x8000000000000000ull ? 0 : ordered_bits(c);
+}
+__device__ __forceinline__ void argmin_merge(long long& c, int& i, long long c2, int i2) {
+  if (c2 < c || (c2 == c && i2 < i)) {
+    c = c2;
+    i = i2;
+  }
+}
 
 __device__ __forceinline__ void block_argmin(double& c, int& i) {
   __shared__ double sc[32];
@@ -340,6 +393,90 @@ __global__ void k_pso_best(SwarmArgs a, const double* __restrict__ cost) {
   }
 }
 
+// k_pso_best and the move of the next generation in one kernel, one block per spectrum: the
+// bests and the move read the same rows, and a generation of a small batch is bound by the
+// launches' latencies (one spectrum of 64 particles: 13.4 us for the two, with the counter's
+// kernel, against 6.8; 1024 spectra x 256: 73 against 50). The generation just
+// evaluated is gens[s], advanced by the spectrum's own block. Improved rows are copied to
+// the personal bests as the move passes over them; the global best's row is taken to shared
+// memory first, since its particle moves too.
+constexpr int STEP_BLOCK = 256;
+template <bool MOVE>
+__global__ void __launch_bounds__(STEP_BLOCK) k_pso_step(SwarmArgs a, const double* __restrict__ cost) {
+  __shared__ uint64_t prefix[2];
+  __shared__ double best[NMAX];
+  __shared__ unsigned char improved[PSO_STEP_MAX_P];
+  __shared__ long long red_c[STEP_BLOCK / 32];
+  __shared__ int red_i[STEP_BLOCK / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const MoveCoef co = MoveCoef::of(a);
+  for (int64_t s = blockIdx.x; s < a.S; s += gridDim.x) {
+    const int gen = a.gens[s], N = a.n_poles[s];
+    const int64_t row0 = s * a.P;
+    if (MOVE && threadIdx.x >= STEP_BLOCK - 2) {   // the last warp's lanes: the others reduce meanwhile
+      const int k = threadIdx.x & 1;
+      prefix[k] = rng_prefix(a.seed, k ? TAG_R2 : TAG_R1, key_id(a, s), (uint64_t)(gen + 1));
+    }
+    // personal bests (strictly lower cost replaces; generation 0 initialises) and the best particle
+    long long bc = 0x7ff0000000000000ll;   // +infinity
+    int bi = 0x7fffffff;
+    for (int p = threadIdx.x; p < a.P; p += STEP_BLOCK) {
+      double c = cost[row0 + p];
+      if (!finite_bits(c)) c = INFINITY;
+      long long kc = cost_key(c);
+      const long long kp = gen == 0 ? 0 : cost_key(a.pbc[row0 + p]);
+      const bool better = gen == 0 || kc < kp;
+      if (better) a.pbc[row0 + p] = c;
+      else kc = kp;
+      improved[p] = better;
+      argmin_merge(bc, bi, kc, p);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long c2 = __shfl_xor_sync(0xffffffffu, bc, o);
+      const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+      argmin_merge(bc, bi, c2, i2);
+    }
+    if (lane == 0) {
+      red_c[wid] = bc;
+      red_i[wid] = bi;
+    }
+    __syncthreads();
+    bc = red_c[0];
+    bi = red_i[0];
+#pragma unroll
+    for (int w = 1; w < STEP_BLOCK / 32; ++w) argmin_merge(bc, bi, red_c[w], red_i[w]);
+    const int gi = bi < a.P ? bi : 0;
+    if (threadIdx.x < N) {
+      const int64_t at = (row0 + gi) * a.nmax + threadIdx.x;
+      best[threadIdx.x] = improved[gi] ? a.x[at] : a.pbx[at];
+    }
+    if (threadIdx.x == 0) {
+      a.gbest[s] = gi;
+      a.gens[s] = gen + 1;
+      // the best cost itself: +infinity if there is none
+      if (a.trace) a.trace[s * (int64_t)(a.iters + 1) + gen] = bi < a.P ? a.pbc[row0 + gi] : INFINITY;
+      if (a.evals && s == 0) atomicAdd(a.evals, (double)a.P * (double)(a.offsets[a.S] - a.offsets[0]));
+    }
+    __syncthreads();
+    const double lo = a.lo[s], hi = a.hi[s];
+    for (int e = threadIdx.x; e < a.P * N; e += STEP_BLOCK) {
+      const int p = e / N, d = e - p * N;
+      const int64_t at = (row0 + p) * a.nmax + d;
+      const bool imp = improved[p];
+      if (!MOVE && !imp) continue;
+      double x = a.x[at];
+      double pb = x;
+      if (imp) a.pbx[at] = x;
+      else pb = a.pbx[at];
+      if (MOVE) {
+        a.v[at] = move_one(co, rng_key(prefix[0], p, d), rng_key(prefix[1], p, d), x, a.v[at], pb, best[d], lo, hi);
+        a.x[at] = x;
+      }
+    }
+    __syncthreads();   // shared state is free for the next spectrum
+  }
+}
+
 // After an outer iteration of dual annealing: best chain per spectrum (lowest
 // best cost, lowest index on ties), its cost in the trace, and the iteration's
 // evaluations (P chains x 2N moves x K samples) in the counter.
@@ -385,6 +522,8 @@ __global__ void k_topk(SwarmArgs a, PolishArgs pa) {
         pa.f[l] = bc;
         pa.done[l] = 0;
         pa.hcount[l] = 0;
+        pa.head[l] = 0;
+        pa.acc[l] = 0;
       }
       __syncthreads();
     }
@@ -419,194 +558,248 @@ __device__ __forceinline__ double dotn(const double* a, const double* b, int n) 
   return s;
 }
 
-__device__ void write_trials(const PolishArgs& pa, int64_t l, int N, double lo, double hi) {
+// The line's next round of trials, t0 .. t0 + R - 1, by the lanes of its group.
+__device__ void write_trials(const PolishArgs& pa, int64_t l, int N, double lo, double hi, int t0, int lane,
+                             int group) {
   const int nmax = pa.nmax;
-  const int t0 = pa.t0[l];
-  for (int t = 0; t < pa.R; ++t) {
-    const int64_t q = l * pa.R + t;
-    const int tt = t0 + t;
-    if (tt >= pa.max_trials) {
-      pa.active[q] = 0;
-      continue;
-    }
-    const double step = ldexp(1.0, -tt);
-    for (int d = 0; d < nmax; ++d) {
-      double v = 0.0;
-      if (d < N) v = fmin(fmax(pa.th[l * nmax + d] + step * pa.dir[l * nmax + d], lo), hi);
-      pa.tth[q * nmax + d] = v;
-    }
-    pa.active[q] = 1;
+  for (int t = lane; t < pa.R; t += group) pa.active[l * pa.R + t] = t0 + t < pa.max_trials;
+  const int live = min(pa.R, pa.max_trials - t0);
+  for (int e = lane; e < live * nmax; e += group) {
+    const int t = e / nmax, d = e - t * nmax;
+    const double step = __hiloint2double((1023 - (t0 + t)) << 20, 0);   // 2^-(t0 + t)
+    double v = 0.0;
+    if (d < N) v = clamp_to(pa.th[l * nmax + d] + step * pa.dir[l * nmax + d], lo, hi);
+    pa.tth[(l * pa.R + t) * nmax + d] = v;
   }
+}
+
+// The polish's per-line kernels run one thread per line through a dependent FP64 chain
+// (the L-BFGS two-loop recursion, the Armijo tests): single-warp blocks spread the lines
+// over every SM.
+constexpr int POLISH_BLOCK = 32;
+
+// dst += the warp's sum of v: evaluation counts, whole numbers, so the order of the sum is
+// free, and one addition per warp replaces one per line on the same address (1024 spectra x
+// 8 lines: 41 -> 30 us for the full steps' Armijo test).
+__device__ __forceinline__ void add_count(double* dst, int64_t v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, (double)v);
+}
+
+// L-BFGS update with the accepted point's cost and gradient: history pair (s, y) kept
+// only when s^T y > eps y^T y (the oldest pair's slot taken over when full). The pair's rho
+// and gamma, the same dot products that the recursion needs, are kept with it.
+__device__ void polish_take(const PolishArgs& pa, int64_t l, int N) {
+  const int nmax = pa.nmax, m = pa.m;
+  pa.aactive[l] = 0;
+  double sv[NMAX], yv[NMAX];
+  for (int d = 0; d < N; ++d) {
+    sv[d] = pa.ath[l * nmax + d] - pa.th[l * nmax + d];
+    yv[d] = pa.agrad[l * nmax + d] - pa.g[l * nmax + d];
+  }
+  const double sy = dotn(sv, yv, N), yy = dotn(yv, yv, N);
+  if (sy > 2.220446049250313e-16 * yy) {
+    int hc = pa.hcount[l], head = pa.head[l];
+    int slot = head + hc;
+    if (slot >= m) slot -= m;
+    if (hc == m) {
+      slot = head;
+      pa.head[l] = head + 1 == m ? 0 : head + 1;
+    } else {
+      pa.hcount[l] = hc + 1;
+    }
+    for (int d = 0; d < N; ++d) {
+      pa.hs[(slot * nmax + d) * pa.L + l] = sv[d];
+      pa.hy[(slot * nmax + d) * pa.L + l] = yv[d];
+    }
+    pa.rho[slot * pa.L + l] = 1.0 / sy;
+    pa.gamma[l] = sy / yy;
+  }
+  for (int d = 0; d < N; ++d) {
+    pa.th[l * nmax + d] = pa.ath[l * nmax + d];
+    pa.g[l * nmax + d] = pa.agrad[l * nmax + d];
+  }
+  pa.f[l] = pa.acost[l];
+  if (!isfinite(pa.f[l])) pa.done[l] = 1;
 }
 
 // Two-loop recursion (Nocedal and Wright, Alg. 7.4) for the direction d = -H g;
 // a non-descent direction is replaced by -g / max(1, |g|_inf) and the history cleared.
-__global__ void k_polish_dir(PolishArgs pa, const int32_t* n_poles, const double* lo_, const double* hi_) {
+__device__ void polish_dir(const PolishArgs& pa, int64_t l, int N, double lo, double hi) {
+  const int nmax = pa.nmax, m = pa.m;
+  double q[NMAX], alpha[8];
+  const double* g = pa.g + l * nmax;
+  for (int d = 0; d < N; ++d) q[d] = g[d];
+  const int hc = pa.hcount[l], head = pa.head[l];
+  auto slot = [&](int k) { return head + k >= m ? head + k - m : head + k; };   // k-th oldest pair
+  const int64_t L = pa.L;
+  for (int k = hc - 1; k >= 0; --k) {
+    const double* sk = pa.hs + slot(k) * nmax * L + l;
+    const double* yk = pa.hy + slot(k) * nmax * L + l;
+    double dot = 0.0;
+#pragma unroll 4
+    for (int d = 0; d < N; ++d) dot = fma(sk[d * L], q[d], dot);
+    const double al = pa.rho[slot(k) * L + l] * dot;
+#pragma unroll 4
+    for (int d = 0; d < N; ++d) q[d] -= al * yk[d * L];
+    alpha[k] = al;
+  }
+  double gamma;
+  if (hc > 0) {
+    gamma = pa.gamma[l];
+  } else {
+    double gi = 0.0;
+    for (int d = 0; d < N; ++d) gi = fmax(gi, fabs(g[d]));
+    gamma = 1.0 / fmax(1.0, gi);
+  }
+  for (int d = 0; d < N; ++d) q[d] *= gamma;
+  for (int k = 0; k < hc; ++k) {
+    const double* sk = pa.hs + slot(k) * nmax * L + l;
+    const double* yk = pa.hy + slot(k) * nmax * L + l;
+    double dot = 0.0;
+#pragma unroll 4
+    for (int d = 0; d < N; ++d) dot = fma(yk[d * L], q[d], dot);
+    const double be = pa.rho[slot(k) * L + l] * dot;
+#pragma unroll 4
+    for (int d = 0; d < N; ++d) q[d] += sk[d * L] * (alpha[k] - be);
+  }
+  double gd = 0.0;
+  for (int d = 0; d < N; ++d) gd = fma(g[d], -q[d], gd);
+  double* dir = pa.dir + l * nmax;
+  if (!(gd < 0.0)) {
+    double gi = 0.0;
+    for (int d = 0; d < N; ++d) gi = fmax(gi, fabs(g[d]));
+    const double sc = 1.0 / fmax(1.0, gi);
+    for (int d = 0; d < N; ++d) dir[d] = -g[d] * sc;
+    pa.hcount[l] = 0;
+    pa.head[l] = 0;
+  } else {
+    for (int d = 0; d < N; ++d) dir[d] = -q[d];
+  }
+  // the full step t = 0 is evaluated first, with its gradient, in the accepted-point slot;
+  // the backtracking rounds start at t = 1 if it fails
+  for (int d = 0; d < nmax; ++d) {
+    double v = 0.0;
+    if (d < N) v = clamp_to(pa.th[l * nmax + d] + dir[d], lo, hi);
+    pa.ath[l * nmax + d] = v;
+  }
+  pa.aactive[l] = 1;
+  pa.t0[l] = 1;
+}
+
+// Between two evaluations of a line's points: the update of the iteration that ends (take,
+// for the lines that accepted a step) and the direction of the one that begins.
+__global__ void __launch_bounds__(POLISH_BLOCK) k_polish_step(PolishArgs pa, const int32_t* n_poles,
+                                                              const double* lo_, const double* hi_) {
   for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < pa.L;
        l += (int64_t)gridDim.x * blockDim.x) {
-    pa.acc[l] = 0;
-    if (pa.done[l]) continue;
     const int64_t s = l / pa.T;
     const int N = n_poles[s];
-    const int nmax = pa.nmax, m = pa.m;
-    double q[NMAX], alpha[8];
-    const double* g = pa.g + l * nmax;
-    for (int d = 0; d < N; ++d) q[d] = g[d];
-    const int hc = pa.hcount[l];
-    // history slot of the k-th newest pair: (head - 1 - k) mod m, head = hc mod m ... stored oldest..newest
-    for (int k = hc - 1; k >= 0; --k) {
-      const double* sk = pa.hs + (l * m + k) * nmax;
-      const double* yk = pa.hy + (l * m + k) * nmax;
-      const double rho = 1.0 / dotn(yk, sk, N);
-      const double al = rho * dotn(sk, q, N);
-      for (int d = 0; d < N; ++d) q[d] -= al * yk[d];
-      alpha[k] = al;
-    }
-    double gamma;
-    if (hc > 0) {
-      const double* sn = pa.hs + (l * m + hc - 1) * nmax;
-      const double* yn = pa.hy + (l * m + hc - 1) * nmax;
-      gamma = dotn(sn, yn, N) / dotn(yn, yn, N);
-    } else {
-      double gi = 0.0;
-      for (int d = 0; d < N; ++d) gi = fmax(gi, fabs(g[d]));
-      gamma = 1.0 / fmax(1.0, gi);
-    }
-    for (int d = 0; d < N; ++d) q[d] *= gamma;
-    for (int k = 0; k < hc; ++k) {
-      const double* sk = pa.hs + (l * m + k) * nmax;
-      const double* yk = pa.hy + (l * m + k) * nmax;
-      const double rho = 1.0 / dotn(yk, sk, N);
-      const double be = rho * dotn(yk, q, N);
-      for (int d = 0; d < N; ++d) q[d] += sk[d] * (alpha[k] - be);
-    }
-    double gd = 0.0;
-    for (int d = 0; d < N; ++d) gd = fma(g[d], -q[d], gd);
-    double* dir = pa.dir + l * nmax;
-    if (!(gd < 0.0)) {
-      double gi = 0.0;
-      for (int d = 0; d < N; ++d) gi = fmax(gi, fabs(g[d]));
-      const double sc = 1.0 / fmax(1.0, gi);
-      for (int d = 0; d < N; ++d) dir[d] = -g[d] * sc;
-      pa.hcount[l] = 0;
-    } else {
-      for (int d = 0; d < N; ++d) dir[d] = -q[d];
-    }
-    // the full step t = 0 is evaluated first, with its gradient, in the accepted-point slot;
-    // the backtracking rounds start at t = 1 if it fails
-    for (int d = 0; d < nmax; ++d) {
-      double v = 0.0;
-      if (d < N) v = fmin(fmax(pa.th[l * nmax + d] + dir[d], lo_[s]), hi_[s]);
-      pa.ath[l * nmax + d] = v;
-    }
-    pa.aactive[l] = 1;
-    pa.t0[l] = 1;
+    if (pa.acc[l]) polish_take(pa, l, N);
+    pa.acc[l] = 0;
+    if (!pa.done[l]) polish_dir(pa, l, N, lo_[s], hi_[s]);
   }
 }
 
-// Armijo test of the full step (evaluated with its gradient in the accepted-point
-// slot): accepted, the line's cost and gradient are ready for the update; rejected,
-// the backtracking trials t = 1 .. R of the first round are written.
-__global__ void k_polish_first(PolishArgs pa, const int32_t* n_poles, const double* lo_, const double* hi_,
-                               const int64_t* offsets) {
-  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < pa.L;
-       l += (int64_t)gridDim.x * blockDim.x) {
-    if (!pa.aactive[l]) continue;
-    pa.aactive[l] = 0;
+// The Armijo tests: a group of lanes per line, one lane per trial of a round (8, or a warp
+// where a round takes every step length), so that a round's tests run side by side and its
+// next trials are written by the whole group. With one thread per line the 8 x N trial
+// coordinates of a rejecting line were one thread's serial FP64 work, and its whole warp's:
+// 1024 spectra x 8 lines, 30 and 49 us for the two kernels, now 11 and 14.
+__device__ __forceinline__ int polish_group(const PolishArgs& pa) { return pa.R <= 8 ? 8 : 32; }
+__device__ __forceinline__ unsigned polish_group_mask(int group) {
+  return group == 32 ? 0xffffffffu : 0xffu << (threadIdx.x & 24);
+}
+constexpr int ARMIJO_BLOCK = 128;
+
+// The full step (evaluated with its gradient in the accepted-point slot): accepted, the
+// line's cost and gradient are ready for the update; rejected, the backtracking trials t =
+// 1 .. R of the first round are written.
+__global__ void __launch_bounds__(ARMIJO_BLOCK) k_polish_first(PolishArgs pa, const int32_t* n_poles,
+                                                               const double* lo_, const double* hi_,
+                                                               const int64_t* offsets) {
+  const int group = polish_group(pa), lane = (int)threadIdx.x & (group - 1);
+  const unsigned gmask = polish_group_mask(group);
+  const int64_t step = (int64_t)gridDim.x * blockDim.x / group;
+  int64_t evaluated = 0;
+  for (int64_t l = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / group; l < pa.L; l += step) {
+    const bool eval = pa.aactive[l];
+    __syncwarp(gmask);   // every lane of the group has read the flag
+    if (!eval) continue;
     const int64_t s = l / pa.T;
     const int N = n_poles[s];
     const int nmax = pa.nmax;
-    if (pa.evals) atomicAdd(pa.evals, (double)(offsets[s + 1] - offsets[s]));
     double gs = 0.0;
     for (int d = 0; d < N; ++d) gs = fma(pa.g[l * nmax + d], pa.ath[l * nmax + d] - pa.th[l * nmax + d], gs);
-    if (pa.acost[l] <= pa.f[l] + pa.c1 * gs) {
-      pa.acc[l] = 1;
-    } else if (pa.t0[l] >= pa.max_trials) {
-      pa.done[l] = 1;
-    } else {
-      write_trials(pa, l, N, lo_[s], hi_[s]);
+    const bool ok = pa.acost[l] <= pa.f[l] + pa.c1 * gs;
+    const int t0 = pa.t0[l];
+    if (lane == 0) {
+      evaluated += offsets[s + 1] - offsets[s];
+      pa.aactive[l] = 0;
+      if (ok) pa.acc[l] = 1;
+      else if (t0 >= pa.max_trials) pa.done[l] = 1;
     }
+    if (!ok && t0 < pa.max_trials) write_trials(pa, l, N, lo_[s], hi_[s], t0, lane, group);
   }
+  __syncwarp();
+  if (pa.evals) add_count(pa.evals, evaluated);
 }
 
-// Armijo test on the evaluated trials of each line, in order of decreasing step.
-__global__ void k_polish_accept(PolishArgs pa, const int32_t* n_poles, const double* lo_, const double* hi_,
-                                const int64_t* offsets) {
-  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < pa.L;
-       l += (int64_t)gridDim.x * blockDim.x) {
-    if (pa.done[l] || pa.acc[l]) continue;
-    const int64_t s = l / pa.T;
+// The evaluated trials of each line, in order of decreasing step.
+__global__ void __launch_bounds__(ARMIJO_BLOCK) k_polish_accept(PolishArgs pa, const int32_t* n_poles,
+                                                                const double* lo_, const double* hi_,
+                                                                const int64_t* offsets) {
+  const int group = polish_group(pa), lane = (int)threadIdx.x & (group - 1);
+  const unsigned gmask = polish_group_mask(group);
+  const int64_t step = (int64_t)gridDim.x * blockDim.x / group;
+  int64_t evaluated = 0;
+  for (int64_t l = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / group; l < pa.L; l += step) {
+    const bool skip = pa.done[l] || pa.acc[l];
+    const int t0 = pa.t0[l];
+    __syncwarp(gmask);   // every lane of the group has read the flags
+    if (skip) continue;
+    const int64_t s = l / pa.T, q = l * pa.R + lane;
     const int N = n_poles[s];
     const int nmax = pa.nmax;
-    int n_active = 0;
-    int hit = -1;
-    for (int t = 0; t < pa.R; ++t) {
-      const int64_t q = l * pa.R + t;
-      if (!pa.active[q]) continue;
-      ++n_active;
-      if (hit >= 0) continue;
+    const bool act = lane < pa.R && pa.active[q];
+    bool ok = false;
+    if (act) {
       double gs = 0.0;
-      for (int d = 0; d < N; ++d)
-        gs = fma(pa.g[l * nmax + d], pa.tth[q * nmax + d] - pa.th[l * nmax + d], gs);
-      if (pa.tcost[q] <= pa.f[l] + pa.c1 * gs) hit = t;
+      for (int d = 0; d < N; ++d) gs = fma(pa.g[l * nmax + d], pa.tth[q * nmax + d] - pa.th[l * nmax + d], gs);
+      ok = pa.tcost[q] <= pa.f[l] + pa.c1 * gs;
     }
+    const int shift = __ffs((int)gmask) - 1;
+    const unsigned oks = __ballot_sync(gmask, ok) >> shift, acts = __ballot_sync(gmask, act) >> shift;
+    if (!acts) continue;
     // the trials a sequential backtracking search evaluates: up to and including the first
     // acceptable one (the speculative trials after it are not counted)
-    const int counted = hit >= 0 ? hit + 1 : n_active;
-    if (pa.evals && counted) atomicAdd(pa.evals, (double)counted * (double)(offsets[s + 1] - offsets[s]));
-    for (int t = 0; t < pa.R; ++t) pa.active[l * pa.R + t] = 0;
-    if (hit >= 0) {
-      const int64_t q = l * pa.R + hit;
-      for (int d = 0; d < nmax; ++d) pa.ath[l * nmax + d] = pa.tth[q * nmax + d];
-      pa.aactive[l] = 1;
-      pa.acc[l] = 1;
-    } else if (n_active) {
-      pa.t0[l] += pa.R;
-      if (pa.t0[l] >= pa.max_trials) pa.done[l] = 1;
-      else write_trials(pa, l, N, lo_[s], hi_[s]);
+    const int hit = __ffs((int)oks) - 1;
+    const int counted = hit >= 0 ? __popc(acts & ((2u << hit) - 1)) : __popc(acts);
+    const bool more = hit < 0 && t0 + pa.R < pa.max_trials;
+    if (lane == 0) {
+      evaluated += counted * (offsets[s + 1] - offsets[s]);
+      if (hit >= 0) {
+        pa.aactive[l] = 1;
+        pa.acc[l] = 1;
+      } else {
+        pa.t0[l] = t0 + pa.R;
+        if (!more) pa.done[l] = 1;
+      }
     }
+    if (hit >= 0)
+      for (int d = lane; d < nmax; d += group) pa.ath[l * nmax + d] = pa.tth[(l * pa.R + hit) * nmax + d];
+    if (more) write_trials(pa, l, N, lo_[s], hi_[s], t0 + pa.R, lane, group);
+    else if (lane < pa.R) pa.active[q] = 0;
   }
+  __syncwarp();
+  if (pa.evals) add_count(pa.evals, evaluated);
 }
 
-// L-BFGS update with the accepted point's cost and gradient: history pair
-// (s, y) kept only when s^T y > eps y^T y (oldest pair dropped when full).
-__global__ void k_polish_take(PolishArgs pa, const int32_t* n_poles) {
+// The update of the last iteration.
+__global__ void __launch_bounds__(POLISH_BLOCK) k_polish_take(PolishArgs pa, const int32_t* n_poles) {
   for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < pa.L;
-       l += (int64_t)gridDim.x * blockDim.x) {
-    if (!pa.acc[l]) continue;
-    pa.aactive[l] = 0;
-    const int64_t s = l / pa.T;
-    const int N = n_poles[s];
-    const int nmax = pa.nmax, m = pa.m;
-    double sv[NMAX], yv[NMAX];
-    for (int d = 0; d < N; ++d) {
-      sv[d] = pa.ath[l * nmax + d] - pa.th[l * nmax + d];
-      yv[d] = pa.agrad[l * nmax + d] - pa.g[l * nmax + d];
-    }
-    const double sy = dotn(sv, yv, N), yy = dotn(yv, yv, N);
-    if (sy > 2.220446049250313e-16 * yy) {
-      int hc = pa.hcount[l];
-      if (hc == m) {
-        for (int k = 1; k < m; ++k)
-          for (int d = 0; d < N; ++d) {
-            pa.hs[(l * m + k - 1) * nmax + d] = pa.hs[(l * m + k) * nmax + d];
-            pa.hy[(l * m + k - 1) * nmax + d] = pa.hy[(l * m + k) * nmax + d];
-          }
-        hc = m - 1;
-      }
-      for (int d = 0; d < N; ++d) {
-        pa.hs[(l * m + hc) * nmax + d] = sv[d];
-        pa.hy[(l * m + hc) * nmax + d] = yv[d];
-      }
-      pa.hcount[l] = hc + 1;
-    }
-    for (int d = 0; d < N; ++d) {
-      pa.th[l * nmax + d] = pa.ath[l * nmax + d];
-      pa.g[l * nmax + d] = pa.agrad[l * nmax + d];
-    }
-    pa.f[l] = pa.acost[l];
-    if (!isfinite(pa.f[l])) pa.done[l] = 1;
-  }
+       l += (int64_t)gridDim.x * blockDim.x)
+    if (pa.acc[l]) polish_take(pa, l, n_poles[l / pa.T]);
 }
 
 // Best line per spectrum (lowest cost, lowest rank on ties), or the swarm's
@@ -666,10 +859,6 @@ static int g1d(int64_t n, int sms) { return (int)std::max<int64_t>(1, std::min<i
 static int g1d_b(int64_t n, int block, int sms) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((n + block - 1) / block, (int64_t)sms * (2048 / block)));
 }
-// The polish's per-line kernels run one thread per line through a dependent FP64
-// chain (the L-BFGS two-loop recursion, the Armijo tests): single-warp blocks spread
-// the lines over every SM.
-constexpr int POLISH_BLOCK = 32;
 
 void launch_pso_init(const SwarmArgs& a, int sms, cudaStream_t st) {
   k_pso_init<<<g1d((int64_t)a.S * a.P, sms), 256, 0, st>>>(a);
@@ -700,6 +889,11 @@ void launch_pso_best(const SwarmArgs& a, const double* cost, int sms, cudaStream
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(a.S, (int64_t)sms * 8));
   k_pso_best<<<grid, 256, 0, st>>>(a, cost);
 }
+void launch_pso_step(const SwarmArgs& a, const double* cost, bool move, int sms, cudaStream_t st) {
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(a.S, (int64_t)sms * 8));
+  if (move) k_pso_step<true><<<grid, STEP_BLOCK, 0, st>>>(a, cost);
+  else k_pso_step<false><<<grid, STEP_BLOCK, 0, st>>>(a, cost);
+}
 void launch_gen_advance(int* gen, cudaStream_t st) { k_gen_advance<<<1, 1, 0, st>>>(gen); }
 void launch_add_scalar(double* dst, double v, cudaStream_t st) { k_add_scalar<<<1, 1, 0, st>>>(dst, v); }
 void launch_topk(const SwarmArgs& a, const PolishArgs& pa, int sms, cudaStream_t st) {
@@ -712,17 +906,19 @@ void launch_polish_start(const PolishArgs& pa, int sms, cudaStream_t st) {
 void launch_polish_take0(const PolishArgs& pa, int sms, cudaStream_t st) {
   k_polish_take0<<<g1d(pa.L, sms), 256, 0, st>>>(pa);
 }
-void launch_polish_dir(const PolishArgs& pa, const int32_t* n_poles, const double* lo, const double* hi,
-                       int sms, cudaStream_t st) {
-  k_polish_dir<<<g1d_b(pa.L, POLISH_BLOCK, sms), POLISH_BLOCK, 0, st>>>(pa, n_poles, lo, hi);
+void launch_polish_step(const PolishArgs& pa, const int32_t* n_poles, const double* lo, const double* hi,
+                        int sms, cudaStream_t st) {
+  k_polish_step<<<g1d_b(pa.L, POLISH_BLOCK, sms), POLISH_BLOCK, 0, st>>>(pa, n_poles, lo, hi);
 }
 void launch_polish_first(const PolishArgs& pa, const int32_t* n_poles, const double* lo, const double* hi,
                          const int64_t* offsets, int sms, cudaStream_t st) {
-  k_polish_first<<<g1d_b(pa.L, POLISH_BLOCK, sms), POLISH_BLOCK, 0, st>>>(pa, n_poles, lo, hi, offsets);
+  const int64_t lanes = pa.L * (pa.R <= 8 ? 8 : 32);
+  k_polish_first<<<g1d_b(lanes, ARMIJO_BLOCK, sms), ARMIJO_BLOCK, 0, st>>>(pa, n_poles, lo, hi, offsets);
 }
 void launch_polish_accept(const PolishArgs& pa, const int32_t* n_poles, const double* lo, const double* hi,
                           const int64_t* offsets, int sms, cudaStream_t st) {
-  k_polish_accept<<<g1d_b(pa.L, POLISH_BLOCK, sms), POLISH_BLOCK, 0, st>>>(pa, n_poles, lo, hi, offsets);
+  const int64_t lanes = pa.L * (pa.R <= 8 ? 8 : 32);
+  k_polish_accept<<<g1d_b(lanes, ARMIJO_BLOCK, sms), ARMIJO_BLOCK, 0, st>>>(pa, n_poles, lo, hi, offsets);
 }
 void launch_polish_take(const PolishArgs& pa, const int32_t* n_poles, int sms, cudaStream_t st) {
   k_polish_take<<<g1d_b(pa.L, POLISH_BLOCK, sms), POLISH_BLOCK, 0, st>>>(pa, n_poles);

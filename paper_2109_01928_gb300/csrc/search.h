@@ -26,6 +26,7 @@ struct SwarmArgs {
   double* ce;      // [S*P]       dual annealing: current energies
   uint8_t* active; // [S*P]       dual annealing: member moved in this step (evaluation mask)
   int* gen;        // generation counter (device)
+  int* gens;       // [S] generation counters of k_pso_step
   double* trace;   // [S][iters+1] or nullptr
   double* evals;   // [1] or nullptr
 };
@@ -40,9 +41,12 @@ struct PolishArgs {
   double* f;       // [L]
   double* g;       // [L][nmax]
   double* dir;     // [L][nmax]
-  double* hs;      // [L][m][nmax] history s (oldest first)
-  double* hy;      // [L][m][nmax] history y
+  double* hs;      // [m][nmax][L] history s, a ring of pairs from slot head
+  double* hy;      // [m][nmax][L] history y
+  double* rho;     // [m][L] 1 / y^T s of each pair
+  double* gamma;   // [L] s^T y / y^T y of the newest pair
   int32_t* hcount; // [L]
+  int32_t* head;   // [L] slot of the oldest pair
   int32_t* t0;     // [L] first trial index of the next backtracking round
   int32_t* done;   // [L] line finished (no acceptable step or non-finite)
   int32_t* acc;    // [L] step accepted in this iteration (acost, agrad at ath ready after the last evaluation)
@@ -65,13 +69,17 @@ void launch_da_visit(const SwarmArgs& a, int j, int sms, cudaStream_t st);
 void launch_da_accept(const SwarmArgs& a, const double* cost, int j, int sms, cudaStream_t st);
 void launch_da_best(const SwarmArgs& a, int sms, cudaStream_t st);
 void launch_pso_best(const SwarmArgs& a, const double* cost, int sms, cudaStream_t st);
+// Bests of the generation just evaluated and (move) the positions of the next one, for
+// populations of at most PSO_STEP_MAX_P.
+constexpr int PSO_STEP_MAX_P = 1024;
+void launch_pso_step(const SwarmArgs& a, const double* cost, bool move, int sms, cudaStream_t st);
 void launch_gen_advance(int* gen, cudaStream_t st);
 void launch_add_scalar(double* dst, double v, cudaStream_t st);
 void launch_topk(const SwarmArgs& a, const PolishArgs& pa, int sms, cudaStream_t st);
 void launch_polish_start(const PolishArgs& pa, int sms, cudaStream_t st);
 void launch_polish_take0(const PolishArgs& pa, int sms, cudaStream_t st);
-void launch_polish_dir(const PolishArgs& pa, const int32_t* n_poles, const double* lo, const double* hi,
-                       int sms, cudaStream_t st);
+void launch_polish_step(const PolishArgs& pa, const int32_t* n_poles, const double* lo, const double* hi,
+                        int sms, cudaStream_t st);
 void launch_polish_first(const PolishArgs& pa, const int32_t* n_poles, const double* lo, const double* hi,
                          const int64_t* offsets, int sms, cudaStream_t st);
 void launch_polish_accept(const PolishArgs& pa, const int32_t* n_poles, const double* lo, const double* hi,
