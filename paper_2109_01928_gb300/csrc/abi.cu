@@ -181,9 +181,13 @@ int debye_ctx::prep_spectra(const debye_spectra* sp, const Plan& pl, cudaStream_
 int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_grad, cudaStream_t st) {
   if (opt.precision != DEBYE_PREC_MIXED_TABLE || pl.S == 0) return DEBYE_OK;
   const int64_t S = pl.S;
-  std::vector<double> lo(S), hi(S);
-  cudaError_t e = cudaMemcpyAsync(lo.data(), sp->lo, sizeof(double) * S, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(hi.data(), sp->hi, sizeof(double) * S, cudaMemcpyDeviceToHost, st);
+  // the bounds, read back through pinned memory
+  void* hb;
+  int rc;
+  if ((rc = stage_begin(2 * sizeof(double) * S, st, &hb))) return rc;
+  double *lo = (double*)hb, *hi = lo + S;
+  cudaError_t e = cudaMemcpyAsync(lo, sp->lo, sizeof(double) * S, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hi, sp->hi, sizeof(double) * S, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(DEBYE_ECUDA, "reading the bounds: %s", cudaGetErrorString(e));
   std::vector<int64_t> seg0(S);
@@ -202,19 +206,21 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
     if (qn > ((int64_t)1 << 31) - 1) return fail(DEBYE_EINVAL, "column-sum tables: too many nodes");
   }
   qn0[S] = (int32_t)qn;
-  int rc;
-  void *d_seg0, *d_nseg, *d_qn0, *d_th, *d_G, *d_x, *d_coef;
-  if ((rc = named("tab.seg0", sizeof(int64_t) * S, &d_seg0)) || (rc = named("tab.nseg", sizeof(int32_t) * S, &d_nseg)) ||
-      (rc = named("tab.qn0", sizeof(int32_t) * (S + 1), &d_qn0)) ||
+  void *d_plan, *d_th, *d_G, *d_x, *d_coef;
+  const size_t plan_bytes = sizeof(int64_t) * S + sizeof(int32_t) * (2 * S + 1);   // seg0, nseg, qn0
+  if ((rc = named("tab.plan", plan_bytes, &d_plan)) ||
       (rc = named("tab.theta", sizeof(double) * TAB_NODE_N * qn, &d_th)) ||
       (rc = named("tab.G", sizeof(double) * (with_grad ? 4 : 2) * TAB_NODE_N * qn, &d_G)) ||
       (rc = named("tab.x", sizeof(double) * TAB_NODE_N * qn, &d_x)) ||
       (rc = named("tab.coef", sizeof(float2) * TAB_NF * TAB_NC * segs, &d_coef)))
     return rc;
-  e = cudaMemcpyAsync(d_seg0, seg0.data(), sizeof(int64_t) * S, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_nseg, nseg.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_qn0, qn0.data(), sizeof(int32_t) * (S + 1), cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return fail(DEBYE_ECUDA, "uploading the table plan: %s", cudaGetErrorString(e));
+  if ((rc = stage_begin(plan_bytes, st, &hb))) return rc;
+  std::memcpy(hb, seg0.data(), sizeof(int64_t) * S);
+  std::memcpy((char*)hb + sizeof(int64_t) * S, nseg.data(), sizeof(int32_t) * S);
+  std::memcpy((char*)hb + (sizeof(int64_t) + sizeof(int32_t)) * S, qn0.data(), sizeof(int32_t) * (S + 1));
+  if ((rc = stage_send(d_plan, plan_bytes, st))) return rc;
+  const int64_t* d_seg0 = (const int64_t*)d_plan;
+  const int32_t *d_nseg = (const int32_t*)(d_seg0 + S), *d_qn0 = d_nseg + S;
   // node pass: TAB_NODE_N poles per pseudo-candidate, 8 pseudo-candidates x 8 lanes per block
   // (a box of 8 decades has 24 pseudo-candidates: with 16 per block, every second block of a
   // spectrum was half empty: 1132 -> 954 us with the derivatives)
@@ -224,7 +230,7 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
   std::vector<int32_t> qb(qn0.begin(), qn0.end() - 1), qe(qn0.begin() + 1, qn0.end());
   UnitGroups gn;
   build_units(pn, qb, qe, CBN, gn);
-  if ((rc = upload_units(gn, ws_tab_units, st))) return rc;   // synchronises: the host plan may go
+  if ((rc = upload_units(gn, ws_tab_units, st))) return rc;
   EvalArgs an{};
   an.units = (const Unit*)ws_tab_units.p;
   an.n_units = (int)gn.units.size();
@@ -246,51 +252,79 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
   an.status = d_status;
   ProfEntry pe;
   if (prof_on) prof_begin(DEBYE_KERNEL_TABLE, 0.0, st, pe);
-  launch_tab_nodes(S, (const int32_t*)d_qn0, (const int32_t*)d_nseg, sp->lo, (double*)d_th, sms, st);
+  launch_tab_nodes(S, d_qn0, d_nseg, sp->lo, (double*)d_th, sms, st);
   if (an.n_units > 0)
     launch_pass(TAB_NODE_N, with_grad ? PH_SUMSG : PH_SUMS, an, std::max(1, std::min(an.n_units, sms * 16)), CBN * KSN, st);
-  launch_tab_coef(S, (const int32_t*)d_qn0, (const int32_t*)d_nseg, (const int64_t*)d_seg0, (const double*)d_G,
+  launch_tab_coef(S, d_qn0, d_nseg, d_seg0, (const double*)d_G,
                   (const double*)d_x, qn, with_grad, (float2*)d_coef, sms, st);
   if (prof_on) prof_end(pe, st);
   launches += 3;
   tab.coef = (const float2*)d_coef;
-  tab.seg0 = (const int64_t*)d_seg0;
-  tab.nseg = (const int32_t*)d_nseg;
+  tab.seg0 = d_seg0;
+  tab.nseg = d_nseg;
   tab.lo = sp->lo;
   tab_max_seg = *std::max_element(nseg.begin(), nseg.end());
   return check_launch("column-sum tables");
 }
 
-// Units over candidate ranges [qb[s], qe[s]) of each spectrum, grouped by pole
-// bucket and, within a bucket, heaviest first (work ~ K (N+2)^2 per candidate).
+// Units over candidate ranges [qb[s], qe[s]) of each spectrum, grouped by pole bucket and,
+// within a bucket, the spectra with the most samples first.
 void debyefit::build_units(const Plan& pl, const std::vector<int32_t>& qb, const std::vector<int32_t>& qe,
                  int cb, UnitGroups& g) {
-  std::vector<std::vector<Unit>> per(N_BUCKETS);
+  std::vector<std::pair<uint64_t, int64_t>> order(pl.S);   // (bucket, samples descending), spectrum
+  size_t n = 0;
   for (int64_t s = 0; s < pl.S; ++s) {
-    const int N = pl.npol[s];
-    for (int32_t q = qb[s]; q < qe[s]; q += cb) {
-      Unit u;
-      u.s = (int32_t)s;
-      u.q0 = q;
-      u.q1 = std::min(qe[s], q + cb);
-      u.N = N;
-      u.k0 = pl.offs[s];
-      u.k1 = pl.offs[s + 1];
-      per[bucket_of(N)].push_back(u);
+    order[s] = {(uint64_t)bucket_of(pl.npol[s]) << 32 | (uint64_t)(((int64_t)1 << 30) - (pl.offs[s + 1] - pl.offs[s])), s};
+    n += (size_t)((qe[s] - qb[s] + cb - 1) / cb);
+  }
+  std::sort(order.begin(), order.end());
+  g.units.resize(n);
+  Unit* u = g.units.data();
+  int b = 0;
+  g.begin[0] = 0;
+  for (const auto& o : order) {
+    const int64_t s = o.second;
+    while (b < bucket_of(pl.npol[s])) g.begin[++b] = (int)(u - g.units.data());
+    for (int32_t q = qb[s]; q < qe[s]; q += cb)
+      *u++ = Unit{(int32_t)s, q, std::min(qe[s], q + cb), pl.npol[s], pl.offs[s], pl.offs[s + 1]};
+  }
+  while (b < N_BUCKETS) g.begin[++b] = (int)(u - g.units.data());
+}
+
+int debye_ctx::stage_begin(size_t bytes, cudaStream_t st, void** host) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(st, &cs);
+  if (e == cudaSuccess && cs != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+  if (e != cudaSuccess) return fail(DEBYE_ECUDA, "uploading a plan: %s", cudaGetErrorString(e));
+  stage_next = (stage_next + 1) % STAGE_SLOTS;
+  StageSlot& s = stage[stage_next];
+  if (s.busy && (e = cudaEventSynchronize(s.ev)) != cudaSuccess)
+    return fail(DEBYE_ECUDA, "uploading a plan: %s", cudaGetErrorString(e));
+  s.busy = false;
+  if (s.cap < bytes) {
+    if (s.own) cudaFreeHost(s.p);
+    s.p = nullptr;
+    s.cap = 0;
+    s.own = false;
+    if (cudaMallocHost(&s.p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      s.p = nullptr;
+      return fail(DEBYE_ENOMEM, "allocation of %zu pinned bytes failed", bytes);
     }
+    s.cap = bytes;
+    s.own = true;
   }
-  g.units.clear();
-  for (int b = 0; b < N_BUCKETS; ++b) {
-    auto& v = per[b];
-    std::stable_sort(v.begin(), v.end(), [](const Unit& x, const Unit& y) {
-      const double wx = (double)(x.k1 - x.k0) * (x.q1 - x.q0) * (x.N + 2) * (x.N + 2);
-      const double wy = (double)(y.k1 - y.k0) * (y.q1 - y.q0) * (y.N + 2) * (y.N + 2);
-      return wx > wy;
-    });
-    g.begin[b] = (int)g.units.size();
-    g.units.insert(g.units.end(), v.begin(), v.end());
-  }
-  g.begin[N_BUCKETS] = (int)g.units.size();
+  *host = s.p;
+  return DEBYE_OK;
+}
+
+int debye_ctx::stage_send(void* dst, size_t bytes, cudaStream_t st) {
+  StageSlot& s = stage[stage_next];
+  cudaError_t e = cudaMemcpyAsync(dst, s.p, bytes, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaEventRecord(s.ev, st);
+  if (e != cudaSuccess) return fail(DEBYE_ECUDA, "uploading a plan: %s", cudaGetErrorString(e));
+  s.busy = true;
+  return DEBYE_OK;
 }
 
 int debye_ctx::upload_units(const UnitGroups& g, Buf& dst, cudaStream_t st) {
@@ -298,11 +332,10 @@ int debye_ctx::upload_units(const UnitGroups& g, Buf& dst, cudaStream_t st) {
   const size_t bytes = sizeof(Unit) * std::max<size_t>(g.units.size(), 1);
   if ((rc = ensure(dst, bytes, "units"))) return rc;
   if (g.units.empty()) return DEBYE_OK;
-  cudaError_t e = cudaMemcpyAsync(dst.p, g.units.data(), sizeof(Unit) * g.units.size(),
-                                  cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return fail(DEBYE_ECUDA, "uploading work units: %s", cudaGetErrorString(e));
-  return DEBYE_OK;
+  void* host;
+  if ((rc = stage_begin(bytes, st, &host))) return rc;
+  std::memcpy(host, g.units.data(), bytes);
+  return stage_send(dst.p, bytes, st);
 }
 
 int debye_ctx::ensure_scratch(int64_t Q, int nmax, ScratchBufs& sb, Scratch& sc) {
@@ -350,34 +383,36 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
   // The buckets are launched from the fewest poles up: measured on a whole mixed_1024
   // fit step (graphs on), this order is 12-15 % faster than launching the most poles
   // first (and for the table precision's solves alone: fits 71.8 ms against 76.2).
+  // A captured pass has a stream per bucket. Launched directly, each further stream costs
+  // two event records and two waits on the host, which at 20 buckets outweighed the
+  // launches: six streams in turn (61 spectra x 37 candidates, N 1-20: 143 us a call against
+  // 153 with one per bucket, 175 with four; 1024 x 256, N 2-12: 1497, 1563 and 1654 us).
   auto fork_buckets = [&](int kind, double flops, int b_hi, auto body) -> int {
-    int first = -1, n_nonempty = 0;
-    for (int b = 0; b < b_hi; ++b)
-      if (g.begin[b + 1] > g.begin[b]) {
-        if (first < 0) first = b;
-        ++n_nonempty;
-      }
+    int n_nonempty = 0;
+    for (int b = 0; b < b_hi; ++b) n_nonempty += g.begin[b + 1] > g.begin[b];
     if (!n_nonempty) return DEBYE_OK;
     ProfEntry pe;
     if (prof_on && kind >= 0) prof_begin(kind, flops, st, pe);
-    const bool fork = n_nonempty > 1;
-    if (fork) cudaEventRecord(ev_fork, st);
+    const int lanes = std::min(n_nonempty, capturing_stream ? N_BUCKETS : 6);
+    if (lanes > 1) {
+      for (int i = 1; i < lanes; ++i)
+        if (int rc = side_stream(i)) return rc;
+      cudaEventRecord(ev_fork, st);
+      for (int i = 1; i < lanes; ++i) cudaStreamWaitEvent(side[i], ev_fork, 0);
+    }
+    int turn = 0;
     for (int b = 0; b < b_hi; ++b) {
       const int n = g.begin[b + 1] - g.begin[b];
       if (!n) continue;
-      cudaStream_t bs = st;
-      if (fork && b != first) {
-        bs = side[b];
-        cudaStreamWaitEvent(bs, ev_fork, 0);
-      }
+      const int i = turn++ % lanes;
       EvalArgs ab = a;
       ab.units = a.units + g.begin[b];
       ab.n_units = n;
-      body(b, ab, bs);
-      if (bs != st) {
-        cudaEventRecord(ev_join[b], bs);
-        cudaStreamWaitEvent(st, ev_join[b], 0);
-      }
+      body(b, ab, i ? side[i] : st);
+    }
+    for (int i = 1; i < lanes; ++i) {
+      cudaEventRecord(ev_join[i], side[i]);
+      cudaStreamWaitEvent(st, ev_join[i], 0);
     }
     if (prof_on && kind >= 0) prof_end(pe, st);
     return check_launch("pass");
@@ -554,11 +589,29 @@ static int eval_entry(debye_handle h, const debye_spectra* sp, int32_t P, int32_
 int debye_ctx::eval_steps(bool) const { return opt.refine_steps; }
 
 
-static bool create_side_streams(debye_ctx* h) {
+int debye_ctx::side_stream(int i) {
+  if (side[i]) return DEBYE_OK;
+  if (cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&ev_join[i], cudaEventDisableTiming) != cudaSuccess)
+    return fail(DEBYE_ECUDA, "side stream: %s", cudaGetErrorString(cudaGetLastError()));
+  return DEBYE_OK;
+}
+
+int debye_ctx::side_streams(const UnitGroups& g) {
+  int n = 0;
   for (int b = 0; b < N_BUCKETS; ++b)
-    if (cudaStreamCreateWithFlags(&h->side[b], cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&h->ev_join[b], cudaEventDisableTiming) != cudaSuccess)
-      return false;
+    if (g.begin[b + 1] > g.begin[b] && n++ > 0)
+      if (int rc = side_stream(n - 1)) return rc;
+  return DEBYE_OK;
+}
+
+static bool create_staging(debye_ctx* h) {
+  if (cudaMallocHost(&h->stage_slab, STAGE_SLOTS * STAGE_SLOT_BYTES) != cudaSuccess) return false;
+  for (int i = 0; i < STAGE_SLOTS; ++i) {
+    h->stage[i].p = (char*)h->stage_slab + i * STAGE_SLOT_BYTES;
+    h->stage[i].cap = STAGE_SLOT_BYTES;
+    if (cudaEventCreateWithFlags(&h->stage[i].ev, cudaEventDisableTiming) != cudaSuccess) return false;
+  }
   return true;
 }
 
@@ -633,7 +686,7 @@ int debye_fit_init(debye_handle* out, const debye_options* opt) {
       cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-      !create_side_streams(h)) {
+      !create_staging(h)) {
     cudaGetLastError();
     h->release();
     delete h;
@@ -762,6 +815,7 @@ int debye_autotune(debye_handle h, const debye_spectra* sp, int32_t P, int32_t n
         int r = setup_eval(h, sp, Pe, n_max, th, c, gr != nullptr, nullptr, set[li], st, es);
         if (r) return r;
         if ((r = run_setup(h, es, c, nullptr, gr, st))) return r;   // untimed: first launch of each kernel
+        if ((r = h->side_streams(es.g))) return r;
         // captured and replayed on the handle's own stream (the caller's may be the legacy
         // default stream, which cannot be captured), ordered after the caller's work
         const cudaStream_t ws = h->work_stream;

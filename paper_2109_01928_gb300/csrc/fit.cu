@@ -106,6 +106,7 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
   UnitGroups g;
   build_units(pl, qb, qe, cb, g);
   if ((rc = h->upload_units(g, h->ws_units, st))) return rc;
+  if ((rc = h->side_streams(g))) return rc;   // before any capture
   EvalArgs ea{};
   if ((rc = h->ensure_scratch(Q, nmax, h->sb_eval, ea.sc))) return rc;
   SwarmArgs sa{};

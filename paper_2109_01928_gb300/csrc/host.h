@@ -30,6 +30,18 @@ struct UnitGroups {
   int begin[N_BUCKETS + 1] = {0};
 };
 
+// Pinned host memory that plans are written to and copied from: a slot's memory may be
+// written again once the copy out of it has run (ev).
+struct StageSlot {
+  void* p = nullptr;
+  size_t cap = 0;
+  bool own = false;      // allocated for this slot (else part of the handle's slab)
+  bool busy = false;     // a copy has been enqueued since the last wait
+  cudaEvent_t ev = nullptr;
+};
+constexpr int STAGE_SLOTS = 4;
+constexpr size_t STAGE_SLOT_BYTES = 256 << 10;   // initial size of each
+
 struct ScratchBufs {
   Buf G, L, vec, rt, fail;
   double* g1 = nullptr;
@@ -63,12 +75,15 @@ struct debye_ctx {
 
   cudaStream_t work_stream = nullptr;  // non-blocking stream of debye_fit_batch
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-  // Pole buckets of one pass run concurrently: bucket b > first on side[b], forked
-  // from and joined back to the launching stream (so their tails overlap).
+  // Pole buckets of one pass run concurrently on side streams forked from and joined back to
+  // the launching stream (so their tails overlap); created as they are first needed.
   cudaStream_t side[debyefit::N_BUCKETS] = {nullptr};
   cudaEvent_t ev_fork = nullptr, ev_join[debyefit::N_BUCKETS] = {nullptr};
 
   debyefit::Buf ws_kq, ws_h0, ws_units;
+  void* stage_slab = nullptr;
+  debyefit::StageSlot stage[debyefit::STAGE_SLOTS];
+  int stage_next = 0;
   debyefit::Buf ws_tab_units;    // units of the column-sum tables' node pass
   debyefit::TabView tab{};       // column-sum tables of the current call (DEBYE_PREC_MIXED_TABLE)
   int tab_max_seg = 0;           // the most segments of a spectrum
@@ -102,6 +117,13 @@ struct debye_ctx {
   int load_plan(const debye_spectra* sp, debyefit::Plan& pl, cudaStream_t st);
   int prep_spectra(const debye_spectra* sp, const debyefit::Plan& pl, cudaStream_t st);
   int upload_units(const debyefit::UnitGroups& g, debyefit::Buf& dst, cudaStream_t st);
+  // A host plan on its way to the device without waiting for the stream: stage_begin gives
+  // `bytes` of pinned memory to write (refused while st is being captured: a replay would
+  // copy whatever the memory holds by then), stage_send enqueues its copy to dst on st.
+  int stage_begin(size_t bytes, cudaStream_t st, void** host);
+  int stage_send(void* dst, size_t bytes, cudaStream_t st);
+  int side_stream(int i);   // create side[i] and its event if need be
+  int side_streams(const debyefit::UnitGroups& g);   // those of a captured pass over g
   int ensure_scratch(int64_t Q, int nmax, debyefit::ScratchBufs& sb, debyefit::Scratch& sc);
   int run_eval(debyefit::EvalArgs a, const debyefit::UnitGroups& g, bool mixed, int steps,
                double* cost, double* weights, double* grad, double* g1, int cb, cudaStream_t st);
@@ -147,6 +169,14 @@ struct debye_ctx {
       ev_join[b] = nullptr;
       side[b] = nullptr;
     }
+    for (debyefit::StageSlot& s : stage) {
+      if (s.busy) cudaEventSynchronize(s.ev);
+      if (s.own) cudaFreeHost(s.p);
+      if (s.ev) cudaEventDestroy(s.ev);
+      s = debyefit::StageSlot{};
+    }
+    if (stage_slab) cudaFreeHost(stage_slab);
+    stage_slab = nullptr;
     if (work_stream) cudaStreamDestroy(work_stream);
     ev_in = ev_out = nullptr;
     work_stream = nullptr;
