@@ -167,7 +167,7 @@ int debye_ctx::prep_spectra(const debye_spectra* sp, const Plan& pl, cudaStream_
   launch_prep(pl.n_samples, pl.S, sp->offsets, sp->omega, sp->eps_re, sp->eps_im, sp->lo, sp->hi,
               (float4*)ws_kq.p, (float4*)ws_kq.p + pl.n_samples, (float4*)ws_kq.p + 2 * pl.n_samples,
               (float4*)ws_kq.p + 3 * pl.n_samples, (double*)ws_h0.p, d_status, sms, st);
-  launches += (pl.n_samples > 0) + (pl.S > 0);
+  launches += pl.S > 0 ? (prep_merged(pl.n_samples, pl.S) ? 1 : 2) : 0;
   return check_launch("prep");
 }
 

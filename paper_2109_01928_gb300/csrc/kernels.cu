@@ -11,30 +11,43 @@ namespace debyefit {
 
 // ------------------------------------------------------------------ input preparation
 // Per sample: float-float splits of (omega 2^-30)^2, eps' and omega eps'' for the column
-// sums (the planes of EvalArgs), and finiteness checks; per spectrum: h0 = sum_k eps'_k
-// and b^T b (FP64).
-__global__ void k_prep_samples(int64_t n, const double* __restrict__ omega,
-                               const double* __restrict__ er, const double* __restrict__ ei,
-                               float4* __restrict__ kq0, float4* __restrict__ kq1, float4* __restrict__ kq2,
-                               int* status) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const double w = omega[k], a = er[k], b = ei[k];
+// sums (the planes of EvalArgs), and finiteness checks; per spectrum: the granules, h0 =
+// sum_k eps'_k and b^T b (FP64).
+struct PrepPlanes {
+  float4 *kq0, *kq1, *kq2;
+};
+struct PrepSample {
+  ff w2, e, c;
+  __device__ __forceinline__ PrepSample(double w, double a, double b, int* status) {
     if (!(w > 0.0) || !isfinite(w) || !isfinite(a) || !isfinite(b)) set_status(status, DEBYE_ENOTFINITE);
     const double ws = w * 0x1p-30;
-    const ff w2 = ff_of(ws * ws), e = ff_of(a), c = ff_of(w * b);
-    kq0[k] = make_float4(w2.h, w2.h, w2.l, w2.l);
-    kq1[k] = make_float4(e.h, e.h, e.l, e.l);
-    kq2[k] = make_float4(c.h, c.h, c.l, c.l);
+    w2 = ff_of(ws * ws);
+    e = ff_of(a);
+    c = ff_of(w * b);
   }
+  __device__ __forceinline__ void write(const PrepPlanes& p, int64_t k) const {
+    p.kq0[k] = make_float4(w2.h, w2.h, w2.l, w2.l);
+    p.kq1[k] = make_float4(e.h, e.h, e.l, e.l);
+    p.kq2[k] = make_float4(c.h, c.h, c.l, c.l);
+  }
+};
+
+__global__ void k_prep_samples(int64_t n, const double* __restrict__ omega, const double* __restrict__ er,
+                               const double* __restrict__ ei, PrepPlanes planes, int* status) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+       k += (int64_t)gridDim.x * blockDim.x)
+    PrepSample(omega[k], er[k], ei[k], status).write(planes, k);
 }
 
-// One block per spectrum; each warp's 32 samples of an iteration are one granule.
+// One block per spectrum; each warp's 32 samples of an iteration are one granule. PLANES:
+// the samples' planes are written here too, one launch and one read of the samples for both
+// (a long spectrum would be one block's work, so there k_prep_samples spreads the samples).
+template <bool PLANES>
 __global__ void k_prep_spectra(int64_t S, const int64_t* __restrict__ offsets, const double* __restrict__ omega,
                                const double* __restrict__ er, const double* __restrict__ ei,
                                const double* __restrict__ lo, const double* __restrict__ hi,
                                double* __restrict__ h0, double* __restrict__ bb, float4* __restrict__ kg,
-                               int* status) {
+                               PrepPlanes planes, int* status) {
   static_assert(GRANULE == 32, "a granule is a warp's samples");
   __shared__ double red[32], red2[32];
   for (int64_t s = blockIdx.x; s < S; s += gridDim.x) {
@@ -44,13 +57,14 @@ __global__ void k_prep_spectra(int64_t S, const int64_t* __restrict__ offsets, c
       const int64_t k = k0 + (threadIdx.x & 31);
       float w2lo = INFINITY, w2hi = 0.f, e = 0.f, c = 0.f;   // neutral for the lanes past the spectrum's end
       if (k < b) {
-        const double w = omega[k], r = er[k], i = ei[k], ws = w * 0x1p-30;
+        const double w = omega[k], r = er[k], i = ei[k];
         acc += r;
         acc2 = fma(r, r, fma(i, i, acc2));
-        w2lo = __double2float_rd(ws * ws);
-        w2hi = __double2float_ru(ws * ws);
-        e = __double2float_rn(r);
-        c = __double2float_rn(w * i);
+        const PrepSample smp(w, r, i, status);
+        if (PLANES) smp.write(planes, k);
+        w2lo = w2hi = smp.w2.h;   // the factor of the bounds' test covers its rounding
+        e = smp.e.h;
+        c = smp.c.h;
         if (!(e >= 0.f && e < INFINITY && c >= 0.f && c < INFINITY && w2lo >= 0.f)) e = c = INFINITY;
       }
       for (int o = 16; o > 0; o >>= 1) {
@@ -553,14 +567,16 @@ void launch_prep(int64_t n_samples, int64_t S, const int64_t* offsets, const dou
                  const double* er, const double* ei, const double* lo, const double* hi,
                  float4* kq0, float4* kq1, float4* kq2, float4* kg, double* h0, int* status, int sms,
                  cudaStream_t st) {
-  if (n_samples > 0) {
-    int grid = (int)std::min<int64_t>((n_samples + 255) / 256, (int64_t)sms * 16);
-    k_prep_samples<<<grid, 256, 0, st>>>(n_samples, omega, er, ei, kq0, kq1, kq2, status);
+  const PrepPlanes planes{kq0, kq1, kq2};
+  if (S <= 0) return;
+  const int grid = (int)std::min<int64_t>(S, (int64_t)sms * 8);
+  if (prep_merged(n_samples, S)) {
+    k_prep_spectra<true><<<grid, 256, 0, st>>>(S, offsets, omega, er, ei, lo, hi, h0, h0 + S, kg, planes, status);
+    return;
   }
-  if (S > 0) {
-    int grid = (int)std::min<int64_t>(S, (int64_t)sms * 8);
-    k_prep_spectra<<<grid, 256, 0, st>>>(S, offsets, omega, er, ei, lo, hi, h0, h0 + S, kg, status);
-  }
+  const int sgrid = (int)std::min<int64_t>((n_samples + 255) / 256, (int64_t)sms * 16);
+  k_prep_samples<<<sgrid, 256, 0, st>>>(n_samples, omega, er, ei, planes, status);
+  k_prep_spectra<false><<<grid, 256, 0, st>>>(S, offsets, omega, er, ei, lo, hi, h0, h0 + S, kg, planes, status);
 }
 
 static int grid_for(int n_units, int sms, int per_sm) {

@@ -68,6 +68,8 @@ inline void launch_pass(int N, int phase, const EvalArgs& a, int grid, int block
 
 // kq0, kq1, kq2: [n_samples] each, the sample planes of EvalArgs; kg: [granule_count];
 // h0: [2 S] doubles, sum_k eps'_k per spectrum, then b^T b per spectrum.
+// One launch, or two (prep_merged false): spectra of more than 4096 samples on average.
+inline bool prep_merged(int64_t n_samples, int64_t S) { return n_samples <= 4096 * S; }
 void launch_prep(int64_t n_samples, int64_t S, const int64_t* offsets, const double* omega,
                  const double* er, const double* ei, const double* lo, const double* hi,
                  float4* kq0, float4* kq1, float4* kq2, float4* kg, double* h0, int* status, int sms,
