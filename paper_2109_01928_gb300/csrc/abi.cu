@@ -380,14 +380,17 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
   // duration is that of the pass as it runs, and its FLOPs those of every bucket.
   // body(b, ab, stream) launches bucket b's work (ab: the arguments restricted to its
   // units) for every non-empty bucket below b_hi; kind >= 0 times the whole fork-join.
-  // The buckets are launched from the fewest poles up: measured on a whole mixed_1024
-  // fit step (graphs on), this order is 12-15 % faster than launching the most poles
-  // first (and for the table precision's solves alone: fits 71.8 ms against 76.2).
+  // Order of the launches. In a captured pass from the fewest poles up: whole fits of 1024
+  // spectra take 301 ms so, 339 with the most poles first (table precision 60.7 and 65.1).
+  // Launched directly on six streams, long passes go the other way, so that the longest
+  // blocks do not start last: 1024 x 256 candidates, mixed, 1404 us against 1506, FP64 column
+  // sums 256 x 256 8.57 ms against 9.20; short ones (1024 x 8 with the gradient, 296 us
+  // against 283) and the table's solves do not gain.
   // A captured pass has a stream per bucket. Launched directly, each further stream costs
   // two event records and two waits on the host, which at 20 buckets outweighed the
   // launches: six streams in turn (61 spectra x 37 candidates, N 1-20: 143 us a call against
   // 153 with one per bucket, 175 with four; 1024 x 256, N 2-12: 1497, 1563 and 1654 us).
-  auto fork_buckets = [&](int kind, double flops, int b_hi, auto body) -> int {
+  auto fork_buckets = [&](int kind, double flops, int b_hi, bool long_passes, auto body) -> int {
     int n_nonempty = 0;
     for (int b = 0; b < b_hi; ++b) n_nonempty += g.begin[b + 1] > g.begin[b];
     if (!n_nonempty) return DEBYE_OK;
@@ -401,7 +404,9 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
       for (int i = 1; i < lanes; ++i) cudaStreamWaitEvent(side[i], ev_fork, 0);
     }
     int turn = 0;
-    for (int b = 0; b < b_hi; ++b) {
+    const bool descending = long_passes && !capturing_stream;
+    for (int k = 0; k < b_hi; ++k) {
+      const int b = descending ? b_hi - 1 - k : k;
       const int n = g.begin[b + 1] - g.begin[b];
       if (!n) continue;
       const int i = turn++ % lanes;
@@ -417,6 +422,7 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
     if (prof_on && kind >= 0) prof_end(pe, st);
     return check_launch("pass");
   };
+  const bool by_warp = solve_sums_by_warp(a.sc.Q, opt.solve_lanes, sms);   // mixed precision's solve
   auto pass_flops = [&](int phase) {
     double fl = 0.0;
     if (prof_on && !a.active)
@@ -428,7 +434,7 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
     ++launches;
   };
   auto per_bucket = [&](int phase) -> int {
-    return fork_buckets(pass_kind(phase, a.active != nullptr), pass_flops(phase), N_BUCKETS,
+    return fork_buckets(pass_kind(phase, a.active != nullptr), pass_flops(phase), N_BUCKETS, !mixed || !by_warp,
                         [&](int b, const EvalArgs& ab, cudaStream_t bs) { launch_bucket_pass(phase, b, ab, bs); });
   };
   auto timed = [&](int kind, auto launch) {
@@ -450,10 +456,9 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
     // wanted), then weights, cost and gradient from the exact Gram identity of the
     // Debye columns. With the thread-per-candidate solve every bucket's solve is
     // launched right after the bucket's pass on the bucket's stream; the
-    // warp-per-candidate solve runs after the join. With kernel timing on, the per-N
-    // solves run after the timed pass, timed on their own.
+    // warp-per-candidate solve runs after the join. With kernel timing on, the solves run
+    // after the timed pass, timed on their own.
     const int ph = grad ? PH_SUMSG : PH_SUMS, sph = grad ? PH_SOLVEG : PH_SOLVE;
-    const bool by_warp = solve_sums_by_warp(a.sc.Q, opt.solve_lanes, sms);
     const int nb_n = by_warp ? 0 : N_BUCKETS;   // buckets with a per-N solve
     auto solve_bucket = [&](int b, const EvalArgs& ab, cudaStream_t bs) {
       if (b >= nb_n) return;
@@ -468,18 +473,19 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
       // the sums of every candidate from the tables (one launch), then the solves
       a.tab = tab;
       timed(DEBYE_KERNEL_TABLE_EVAL, [&] { launch_tab_eval(a, grad != nullptr, tab_max_seg, sms, st); });
-      rc = fork_buckets(prof_on ? DEBYE_KERNEL_SOLVE : -1, 0.0, nb_n, solve_bucket);
+      rc = fork_buckets(prof_on ? DEBYE_KERNEL_SOLVE : -1, 0.0, nb_n, false, solve_bucket);
     } else if (!prof_on) {
-      rc = fork_buckets(-1, 0.0, N_BUCKETS, [&](int b, const EvalArgs& ab, cudaStream_t bs) {
+      rc = fork_buckets(-1, 0.0, N_BUCKETS, !by_warp, [&](int b, const EvalArgs& ab, cudaStream_t bs) {
         launch_bucket_pass(ph, b, ab, bs);
         solve_bucket(b, ab, bs);
       });
     } else {
       rc = per_bucket(ph);
-      if (!rc) rc = fork_buckets(DEBYE_KERNEL_SOLVE, 0.0, nb_n, solve_bucket);
+      if (!rc) rc = fork_buckets(DEBYE_KERNEL_SOLVE, 0.0, nb_n, false, solve_bucket);
     }
     if (rc) return rc;
-    if (by_warp) timed(DEBYE_KERNEL_SOLVE, [&] { launch_solve_sums_warp(a, cost, weights, grad, cb, sms, st); });
+    if (by_warp)
+      timed(DEBYE_KERNEL_SOLVE, [&] { launch_solve_sums_warp(a, cost, weights, grad, cb, sms, st); });
     return check_launch("column-sum solve");
   }
   if ((rc = per_bucket(opt.precision == DEBYE_PREC_FP64_SUMS ? PH_GRAM_SUMS : PH_GRAM))) return rc;
