@@ -456,8 +456,9 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
     // wanted), then weights, cost and gradient from the exact Gram identity of the
     // Debye columns. With the thread-per-candidate solve every bucket's solve is
     // launched right after the bucket's pass on the bucket's stream; the
-    // warp-per-candidate solve runs after the join. With kernel timing on, the solves run
-    // after the timed pass, timed on their own.
+    // warp-per-candidate solve is part of the pass in tiny evaluations (fuse_solve) and
+    // else runs after the join. With kernel timing on, the solves run after the timed
+    // pass, timed on their own.
     const int ph = grad ? PH_SUMSG : PH_SUMS, sph = grad ? PH_SOLVEG : PH_SOLVE;
     const int nb_n = by_warp ? 0 : N_BUCKETS;   // buckets with a per-N solve
     auto solve_bucket = [&](int b, const EvalArgs& ab, cudaStream_t bs) {
@@ -475,6 +476,13 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
       timed(DEBYE_KERNEL_TABLE_EVAL, [&] { launch_tab_eval(a, grad != nullptr, tab_max_seg, sms, st); });
       rc = fork_buckets(prof_on ? DEBYE_KERNEL_SOLVE : -1, 0.0, nb_n, false, solve_bucket);
     } else if (!prof_on) {
+      // Up to two blocks per SM the launches are what takes the time (one spectrum's fit
+      // 2.92 -> 2.65 ms); beyond, the solves want more warps per SM than the pass has (1024
+      // spectra x 8 points with the gradient, 4096 units: 288 us apart, 335 in the pass).
+      a.fuse_solve = by_warp && a.n_units <= 2 * sms;
+      a.out_cost = cost;
+      a.out_weights = weights;
+      a.out_grad = grad;
       rc = fork_buckets(-1, 0.0, N_BUCKETS, !by_warp, [&](int b, const EvalArgs& ab, cudaStream_t bs) {
         launch_bucket_pass(ph, b, ab, bs);
         solve_bucket(b, ab, bs);
@@ -484,7 +492,7 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
       if (!rc) rc = fork_buckets(DEBYE_KERNEL_SOLVE, 0.0, nb_n, false, solve_bucket);
     }
     if (rc) return rc;
-    if (by_warp)
+    if (by_warp && !a.fuse_solve)
       timed(DEBYE_KERNEL_SOLVE, [&] { launch_solve_sums_warp(a, cost, weights, grad, cb, sms, st); });
     return check_launch("column-sum solve");
   }

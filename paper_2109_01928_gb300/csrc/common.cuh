@@ -116,10 +116,11 @@ struct EvalArgs {
   const uint8_t* active;   // [Q] optional candidate mask (nullptr: all)
   int32_t* n_failed;       // [S] optional: +1 per evaluated candidate whose damped matrix is not
                            //   positive definite (its cost is +inf)
+  int32_t fuse_solve;      // column-sum pass: solve each unit's candidates (a warp each) as its sums are done
   int32_t sums_f64;        // column-sum pass: write tau and the sums in FP64 (the tables' node pass)
   int32_t ks;              // lanes per candidate in the pass kernels (power of two <= 32)
   double lam;
-  double* out_cost;        // PH_SOLVE / PH_SOLVEG outputs: cost [Q], weights [Q][nmax+1] or
+  double* out_cost;        // PH_SOLVE / PH_SOLVEG and fuse_solve outputs: cost [Q], weights [Q][nmax+1] or
   double* out_weights;     //   nullptr, gradient [Q][nmax] (PH_SOLVEG)
   double* out_grad;
   Scratch sc;

@@ -25,6 +25,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "solve_warp.cuh"
 
 namespace debyefit {
 
@@ -782,10 +783,21 @@ __device__ __forceinline__ void dispatch_n(const EvalArgs& a, const Unit& u) {
 // pole counts compiled into this kernel (the library launches one N per kernel). At most MAXT threads per block; MINB
 // resident blocks of that size bound the registers per thread (128 x 3: 168
 // registers, 12 warps per SM with 64-thread blocks).
+// The solves of a unit's candidates by the block that summed them (fuse_solve, evaluations of
+// a few units): there the launch between the pass and its solve is a good part of the whole.
+// The sums are read back through global memory: the block wrote them, the barrier orders
+// them.
+template <int N, bool GRAD>
+static __device__ __noinline__ void solve_unit(const EvalArgs& a, const Unit& u) {
+  __syncthreads();
+  for (int q = u.q0 + ((int)threadIdx.x >> 5); q < u.q1; q += (int)blockDim.x >> 5)
+    if (!a.active || a.active[q]) warp_solve<N + 1>(a, u, q, a.out_cost, a.out_weights, GRAD ? a.out_grad : nullptr);
+}
+
 // The column-sum pass (PH_SUMS, PH_SUMSG) of pole count N: one block per unit
 // (grid-stride over the unit list), the unit's samples staged by bulk copies.
 template <int N, bool GRAD, int MAXT, int MINB>
-__global__ void __launch_bounds__(MAXT, MINB) k_pass_sums(EvalArgs a) {
+__global__ void __launch_bounds__(MAXT, MINB) k_pass_sums(const __grid_constant__ EvalArgs a) {
   __shared__ __align__(128) float4 stage_buf[STAGE_RECORDS];
   __shared__ __align__(8) uint64_t stage_bar[2];
   Stage st;
@@ -797,6 +809,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_pass_sums(EvalArgs a) {
       continue;
     }
     if (!sums_sq_unit<N, GRAD>(a, u, st)) return;
+    if (a.fuse_solve) solve_unit<N, GRAD>(a, u);
   }
 }
 
