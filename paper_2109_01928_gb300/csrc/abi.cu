@@ -221,10 +221,13 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
   if ((rc = stage_send(d_plan, plan_bytes, st))) return rc;
   const int64_t* d_seg0 = (const int64_t*)d_plan;
   const int32_t *d_nseg = (const int32_t*)(d_seg0 + S), *d_qn0 = d_nseg + S;
-  // node pass: TAB_NODE_N poles per pseudo-candidate, 8 pseudo-candidates x 8 lanes per block
-  // (a box of 8 decades has 24 pseudo-candidates: with 16 per block, every second block of a
-  // spectrum was half empty: 1132 -> 954 us with the derivatives)
-  constexpr int CBN = 8, KSN = 8;
+  // node pass: 16 pseudo-candidates x 8 lanes per block; a box of 8 decades has 80
+  // pseudo-candidates of 6 nodes, 5 full blocks. A cost-only evaluation of 1024 spectra x 256
+  // candidates 721 us, of 4 spectra of 2000 samples 168 us, with the gradient at 16
+  // candidates 1082 and 217 us. With 20 nodes (three and four sweeps one after the other in
+  // a block) and 8 x 8: 756, 261, 1173 and 407 us; 12 nodes, 8 x 8: 731, 199, 1110 and 299;
+  // 8 nodes, 16 x 8, cost only 734 and 181; 6 nodes, 8 x 8, gradient 1093 and 217.
+  constexpr int CBN = 16, KSN = 8;
   Plan pn = pl;
   std::fill(pn.npol.begin(), pn.npol.end(), TAB_NODE_N);
   std::vector<int32_t> qb(qn0.begin(), qn0.end() - 1), qe(qn0.begin() + 1, qn0.end());
@@ -254,7 +257,7 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
   if (prof_on) prof_begin(DEBYE_KERNEL_TABLE, 0.0, st, pe);
   launch_tab_nodes(S, d_qn0, d_nseg, sp->lo, (double*)d_th, sms, st);
   if (an.n_units > 0)
-    launch_pass(TAB_NODE_N, with_grad ? PH_SUMSG : PH_SUMS, an, std::max(1, std::min(an.n_units, sms * 16)), CBN * KSN, st);
+    launch_pass(TAB_NODE_N, with_grad ? PH_SUMSG : PH_SUMS, an, an.n_units, CBN * KSN, st);
   launch_tab_coef(S, d_qn0, d_nseg, d_seg0, (const double*)d_G,
                   (const double*)d_x, qn, with_grad, (float2*)d_coef, sms, st);
   if (prof_on) prof_end(pe, st);

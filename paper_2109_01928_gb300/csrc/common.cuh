@@ -76,7 +76,10 @@ constexpr int TAB_NC = 12;       // Chebyshev coefficients per segment and funct
 // series converges faster still), which the cost needs, then dS/dtheta and dh/dtheta
 // for the gradient.
 constexpr int TAB_NF = 5;
-constexpr int TAB_NODE_N = 20;   // nodes per pseudo-candidate of the table's node pass
+// Nodes per pseudo-candidate of the table's node pass: one sweep of the column-sum pass, with
+// and without the derivative sums (SQUARED_CHUNK_GRAD), so that a spectrum's nodes spread
+// over as many blocks as possible. Times beside the launch (build_tables).
+constexpr int TAB_NODE_N = 6;
 constexpr int TAB_MAX_SEG = 1000;   // segments per spectrum (a box of at most 200 decades)
 
 struct TabView {
