@@ -370,7 +370,7 @@ int debye_ctx::ensure_scratch(int64_t Q, int nmax, ScratchBufs& sb, Scratch& sc)
 }
 
 // The whole evaluation of one candidate set. Mixed precision: the float-float
-// column-sum pass and k_solve_sums (weights, cost and optionally the gradient).
+// column-sum pass and its solve (weights, cost and optionally the gradient).
 // FP64: Gram pass, solve, `steps` residual passes with refinement, flip and
 // cost, and optionally the gradient passes. Units must already be on the device
 // (a.units); a.bb must be set (b^T b per spectrum) for the mixed path.

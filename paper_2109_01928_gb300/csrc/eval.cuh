@@ -11,7 +11,7 @@
 // Mixed precision (float-float on the FP32 pipe):
 //   sums_sq_unit column sums S_i = sum re_i and h = A^T b of the Debye basis (and,
 //                for the gradient, the same sums over the derivative columns),
-//                from which k_solve_sums forms the Gram, weights, cost and gradient.
+//                from which the column-sum solve forms the Gram, weights, cost and gradient.
 // FP64 precision:
 //   gram_unit    G = A^T A (packed, (N+1)x(N+1)) and h = A^T b of the stacked
 //                real basis of Eq. 7 (rows: eps' and eps'' of every sample).
@@ -354,7 +354,7 @@ __device__ __forceinline__ bool stage_wait(const EvalArgs& a, Stage& st, int b) 
 }
 
 // ------------------------------------------------------------------ column-sum pass (mixed)
-// For the mixed evaluation from column sums (k_solve_sums): per candidate, in
+// For the mixed evaluation from column sums (solve_sums.cuh): per candidate, in
 // float-float,
 //   S_i = sum_k re_i(k)                      (the pole block of the Gram follows from these)
 //   h_i = sum_k re_i(k) eps'_k + im_i(k) eps''_k   (A^T b without the eps_inf row)
@@ -779,10 +779,6 @@ __device__ __forceinline__ void dispatch_n(const EvalArgs& a, const Unit& u) {
   }
 }
 
-// One block per unit (grid-stride over the unit list); LO..HI is the range of
-// pole counts compiled into this kernel (the library launches one N per kernel). At most MAXT threads per block; MINB
-// resident blocks of that size bound the registers per thread (128 x 3: 168
-// registers, 12 warps per SM with 64-thread blocks).
 // The solves of a unit's candidates by the block that summed them (fuse_solve, evaluations of
 // a few units): there the launch between the pass and its solve is a good part of the whole.
 // The sums are read back through global memory: the block wrote them, the barrier orders
@@ -813,6 +809,9 @@ __global__ void __launch_bounds__(MAXT, MINB) k_pass_sums(const __grid_constant_
   }
 }
 
+// One block per unit (grid-stride over the unit list); LO..HI is the range of pole counts
+// compiled into this kernel (the library launches one N per kernel). At most MAXT threads
+// per block; MINB resident blocks of that size bound the registers per thread.
 template <int PH, int LO, int HI, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) k_pass(EvalArgs a) {
   for (int ui = blockIdx.x; ui < a.n_units; ui += gridDim.x) {

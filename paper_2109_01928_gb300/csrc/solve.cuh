@@ -8,7 +8,7 @@
 //   M v      = D L (L^T (D v))
 //   v^T M v  = || L^T (D v) ||^2
 // The factor and the products with it are computed in type T (the FP64 path
-// instantiates double; the mixed path solves its systems in k_solve_sums, with
+// instantiates double; the mixed path solves its systems in solve_sums.cuh, with
 // an FP32 copy of the factor refined in float-float).
 #pragma once
 #include "common.cuh"

@@ -1,6 +1,5 @@
-// Mixed-precision weights, cost and gradient from the column sums (one thread per
-// candidate), shared by the general kernel (kernels.cu) and the per-pole-count
-// kernels launched after each bucket's column-sum pass (pass_b*.cu).
+// Mixed-precision weights, cost and gradient from the column sums, one thread per
+// candidate: a kernel per pole count (pass_b*.cu), launched after its column-sum pass.
 #pragma once
 #include "common.cuh"
 

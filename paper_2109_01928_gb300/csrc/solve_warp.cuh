@@ -7,13 +7,13 @@
 namespace debyefit {
 
 // ------------------------------------------------------------------ cost from column sums, a warp per candidate
-// The algebra of k_solve_sums with lane r holding row r of the (N+1)-square
+// The algebra of solve_sums.cuh with lane r holding row r of the (N+1)-square
 // systems, so that its O(N^2) loops run across the lanes: M one row per lane,
 // the factorisation one column per step (rows in parallel), the triangular
 // solves one unknown per step (broadcast by shuffle), the products with M one
 // row per lane and the gradient one pole per lane. It serves evaluations too
 // small to fill the GPU with one thread per candidate (the polish's line-search
-// and accepted points), where k_solve_sums takes the latency of one candidate's
+// and accepted points), where a thread per candidate takes the latency of one candidate's
 // serial solve: latency is all that bounds it. So each lane keeps its rows of M, L
 // and L^T in registers (NP slots, the loops unrolled with a uniform exit at n) and
 // every other lane's value comes by a shuffle that no earlier step delays: the
@@ -190,7 +190,7 @@ __device__ __forceinline__ void warp_solve(const EvalArgs& a, const Unit& u, int
     if (r < nmax) grad[(int64_t)q * nmax + r] = 0.0;
     return;
   }
-  // d cost / d theta_i in lane r = i + 1 (the formula of k_solve_sums)
+  // d cost / d theta_i in lane r = i + 1 (the formula in solve_sums.cuh)
   const ff ln10 = ff_of(2.302585092994046);
   ff ax = ff_prod(Di, shfl_ff(x, 0)), aw = ff_prod(Di, shfl_ff(w, 0)), as = ax;
 #pragma unroll
