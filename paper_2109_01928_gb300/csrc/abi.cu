@@ -206,12 +206,13 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
     if (qn > ((int64_t)1 << 31) - 1) return fail(DEBYE_EINVAL, "column-sum tables: too many nodes");
   }
   qn0[S] = (int32_t)qn;
-  void *d_plan, *d_th, *d_G, *d_x, *d_coef;
+  void *d_plan, *d_th, *d_G, *d_x, *d_done, *d_coef;
   const size_t plan_bytes = sizeof(int64_t) * S + sizeof(int32_t) * (2 * S + 1);   // seg0, nseg, qn0
   if ((rc = named("tab.plan", plan_bytes, &d_plan)) ||
       (rc = named("tab.theta", sizeof(double) * TAB_NODE_N * qn, &d_th)) ||
       (rc = named("tab.G", sizeof(double) * (with_grad ? 4 : 2) * TAB_NODE_N * qn, &d_G)) ||
       (rc = named("tab.x", sizeof(double) * TAB_NODE_N * qn, &d_x)) ||
+      (rc = named("tab.done", sizeof(int32_t) * S, &d_done)) ||
       (rc = named("tab.coef", sizeof(float2) * TAB_NF * TAB_NC * segs, &d_coef)))
     return rc;
   if ((rc = stage_begin(plan_bytes, st, &hb))) return rc;
@@ -221,18 +222,17 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
   if ((rc = stage_send(d_plan, plan_bytes, st))) return rc;
   const int64_t* d_seg0 = (const int64_t*)d_plan;
   const int32_t *d_nseg = (const int32_t*)(d_seg0 + S), *d_qn0 = d_nseg + S;
-  // node pass: 16 pseudo-candidates x 8 lanes per block; a box of 8 decades has 80
+  // node sums: TAB_CB pseudo-candidates x TAB_KS lanes per block; a box of 8 decades has 80
   // pseudo-candidates of 6 nodes, 5 full blocks. A cost-only evaluation of 1024 spectra x 256
   // candidates 721 us, of 4 spectra of 2000 samples 168 us, with the gradient at 16
   // candidates 1082 and 217 us. With 20 nodes (three and four sweeps one after the other in
   // a block) and 8 x 8: 756, 261, 1173 and 407 us; 12 nodes, 8 x 8: 731, 199, 1110 and 299;
   // 8 nodes, 16 x 8, cost only 734 and 181; 6 nodes, 8 x 8, gradient 1093 and 217.
-  constexpr int CBN = 16, KSN = 8;
   Plan pn = pl;
   std::fill(pn.npol.begin(), pn.npol.end(), TAB_NODE_N);
   std::vector<int32_t> qb(qn0.begin(), qn0.end() - 1), qe(qn0.begin() + 1, qn0.end());
   UnitGroups gn;
-  build_units(pn, qb, qe, CBN, gn);
+  build_units(pn, qb, qe, TAB_CB, gn);
   if ((rc = upload_units(gn, ws_tab_units, st))) return rc;
   EvalArgs an{};
   an.units = (const Unit*)ws_tab_units.p;
@@ -245,7 +245,7 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
   an.omega = sp->omega;
   an.eps_re = sp->eps_re;
   an.eps_im = sp->eps_im;
-  an.ks = KSN;
+  an.ks = TAB_KS;
   an.sums_f64 = 1;   // the coefficients are formed in FP64
   an.lam = opt.lam_search;
   an.sc.Q = qn;
@@ -255,13 +255,10 @@ int debye_ctx::build_tables(const debye_spectra* sp, const Plan& pl, bool with_g
   an.status = d_status;
   ProfEntry pe;
   if (prof_on) prof_begin(DEBYE_KERNEL_TABLE, 0.0, st, pe);
-  launch_tab_nodes(S, d_qn0, d_nseg, sp->lo, (double*)d_th, sms, st);
-  if (an.n_units > 0)
-    launch_pass(TAB_NODE_N, with_grad ? PH_SUMSG : PH_SUMS, an, an.n_units, CBN * KSN, st);
-  launch_tab_coef(S, d_qn0, d_nseg, d_seg0, (const double*)d_G,
-                  (const double*)d_x, qn, with_grad, (float2*)d_coef, sms, st);
+  launch_tab_build(an, S, d_qn0, d_nseg, d_seg0, sp->lo, (double*)d_th, (int32_t*)d_done, with_grad,
+                   (float2*)d_coef, sms, st);
   if (prof_on) prof_end(pe, st);
-  launches += 3;
+  launches += 2;
   tab.coef = (const float2*)d_coef;
   tab.seg0 = d_seg0;
   tab.nseg = d_nseg;

@@ -93,14 +93,15 @@ void launch_grad_finish(const EvalArgs& a, double* grad, int block, int sms, cud
 }  // namespace debyefit
 
 namespace debyefit {
-// Column-sum tables (tables.cu, DEBYE_PREC_MIXED_TABLE). Nodes: theta of every node of
-// every spectrum's table into theta_n[qn0[S]][TAB_NODE_N]; coefficients from the node
-// pass's sums G[4 TAB_NODE_N][Qn] and taus X[TAB_NODE_N][Qn]; eval: the units' column sums (and with grad their
-// theta derivatives) from a.tab into a.sc.x / a.sc.G, as the column-sum pass writes them.
-void launch_tab_nodes(int64_t S, const int32_t* qn0, const int32_t* nseg, const double* lo, double* theta_n,
-                      int sms, cudaStream_t st);
-void launch_tab_coef(int64_t S, const int32_t* qn0, const int32_t* nseg, const int64_t* seg0, const double* G,
-                     const double* X, int64_t Qn, bool with_grad, float2* coef, int sms, cudaStream_t st);
+// Column-sum tables (tables.cu, DEBYE_PREC_MIXED_TABLE). Build (2 launches): theta of every
+// node of every spectrum's table into theta_n[qn0[S]][TAB_NODE_N], the nodes' sums over a's
+// units (TAB_CB pseudo-candidates each) into a.sc, the coefficients; done: [S] scratch. Eval:
+// the units' column sums (and with grad their theta derivatives) from a.tab into a.sc.x /
+// a.sc.G, as the column-sum pass writes them.
+constexpr int TAB_CB = 16, TAB_KS = 8;   // node sums: pseudo-candidates of a block, lanes of each
+void launch_tab_build(const EvalArgs& a, int64_t S, const int32_t* qn0, const int32_t* nseg, const int64_t* seg0,
+                      const double* lo, double* theta_n, int32_t* done, bool with_grad, float2* coef, int sms,
+                      cudaStream_t st);
 void launch_tab_eval(const EvalArgs& a, bool grad, int max_seg, int sms, cudaStream_t st);
 // One block running the column-sum pass's bounded staging wait with nothing to wait
 // for (waitcheck.cu): it records DEBYE_ETIMEOUT after the wait's clock budget;

@@ -18,6 +18,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "eval.cuh"
 #include "launch.h"
 
 namespace debyefit {
@@ -49,13 +50,23 @@ static const ChebConst& cheb_const() {
   return c;
 }
 
+struct TabBuild {
+  ChebConst cc;
+  const int32_t* qn0;      // [S + 1] first pseudo-candidate of each spectrum
+  const int32_t* nseg;     // [S]
+  const int64_t* seg0;     // [S]
+  int32_t* done;           // [S] units of the spectrum that have ended
+  float2* coef;
+};
+
 // Node thetas, pseudo-candidate-major: spectrum s owns rows qn0[s] .. qn0[s+1]-1 of
 // theta_n[.][TAB_NODE_N]; node n = g NC + m (segment g, point m) sits at slot n of the
 // spectrum's rows, theta = lo + TAB_W (g + 1/2 + x_m / 2); slots past the last node
-// repeat it.
+// repeat it. Zeroes the spectrum's count of ended units.
 __global__ void k_tab_nodes(int64_t S, const int32_t* qn0, const int32_t* nseg, const double* lo,
-                            ChebConst cc, double* theta_n) {
+                            ChebConst cc, double* theta_n, int32_t* done) {
   for (int64_t s = blockIdx.x; s < S; s += gridDim.x) {
+    if (threadIdx.x == 0) done[s] = 0;
     const int64_t base = (int64_t)qn0[s] * TAB_NODE_N;
     const int slots = (qn0[s + 1] - qn0[s]) * TAB_NODE_N;
     const int nodes = nseg[s] * TAB_NC;
@@ -68,48 +79,73 @@ __global__ void k_tab_nodes(int64_t S, const int32_t* qn0, const int32_t* nseg, 
   }
 }
 
-// Coefficients of segment g and function f of spectrum s from the node pass's output:
-// for node n, pseudo-candidate q = qn0[s] + n / TAB_NODE_N and pole i = n % TAB_NODE_N,
-// the column-sum pass wrote S, h, dS, dh at G[(r TAB_NODE_N + i) Qn + q], r = 0..3, and
-// tau at X[i Qn + q].
-__global__ void k_tab_coef(int64_t S, const int32_t* qn0, const int32_t* nseg, const int64_t* seg0,
-                           ChebConst cc, const double* G, const double* X, int64_t Qn, int nf, float2* coef) {
-  for (int64_t s = blockIdx.x; s < S; s += gridDim.x) {
-    const int items = nseg[s] * nf;   // nf: the functions tabulated, the first 3 or all
-    for (int it = threadIdx.x; it < items; it += blockDim.x) {
-      const int g = it / nf, f = it % nf;
-      double v[TAB_NC];
+// Coefficients of segment g and function f of spectrum s from the node sums: for node n,
+// pseudo-candidate q = qn0[s] + n / TAB_NODE_N and pole i = n % TAB_NODE_N, S, h, dS, dh
+// stand at G[(r TAB_NODE_N + i) Qn + q], r = 0..3, and tau at X[i Qn + q]. Other blocks wrote
+// them: they are read from L2 (a sector that this SM's L1 holds may be older). Called by a
+// whole block; nf: the functions tabulated, the first 3 or all.
+__device__ __forceinline__ void tab_coef(const TabBuild& t, const double* G, const double* X, int64_t Qn, int64_t s,
+                                         int nf) {
+  const ChebConst& cc = t.cc;
+  const int items = t.nseg[s] * nf;
+  for (int it = threadIdx.x; it < items; it += blockDim.x) {
+    const int g = it / nf, f = it % nf;
+    double v[TAB_NC];
 #pragma unroll
-      for (int m = 0; m < TAB_NC; ++m) {
-        const int n = g * TAB_NC + m;
-        const int64_t q = qn0[s] + n / TAB_NODE_N;
-        const int i = n % TAB_NODE_N;
-        v[m] = f == 2 ? X[(int64_t)i * Qn + q] : G[(int64_t)((f < 2 ? f : f - 1) * TAB_NODE_N + i) * Qn + q];
-      }
-      double c[TAB_NC];
+    for (int m = 0; m < TAB_NC; ++m) {
+      const int n = g * TAB_NC + m;
+      const int64_t q = t.qn0[s] + n / TAB_NODE_N;
+      const int i = n % TAB_NODE_N;
+      v[m] = __ldcg(f == 2 ? X + (int64_t)i * Qn + q : G + (int64_t)((f < 2 ? f : f - 1) * TAB_NODE_N + i) * Qn + q);
+    }
+    double c[TAB_NC];
 #pragma unroll
-      for (int k = 0; k < TAB_NC; ++k) {
-        c[k] = 0.0;
+    for (int k = 0; k < TAB_NC; ++k) {
+      c[k] = 0.0;
 #pragma unroll
-        for (int m = 0; m < TAB_NC; ++m) c[k] = fma(cc.dct[k][m], v[m], c[k]);
-      }
-      // monomial coefficients in x (the series' coefficients fall by ~20 a degree, the
-      // Chebyshev polynomials' monomial coefficients grow by at most 1 + sqrt 2: the
-      // monomial form is as well conditioned on [-1, 1]). T_j has only powers of j's parity:
-      // the skipped terms' factors are zero, and with the splits on the integer pipe 72 of
-      // the kernel's 258 FP64 operations (64 cycles per warp each, what bounds it) fall away
-      // without a change of the results.
-      float2* out = coef + ((seg0[s] + g) * TAB_NF + f) * TAB_NC;
+      for (int m = 0; m < TAB_NC; ++m) c[k] = fma(cc.dct[k][m], v[m], c[k]);
+    }
+    // monomial coefficients in x (the series' coefficients fall by ~20 a degree, the
+    // Chebyshev polynomials' monomial coefficients grow by at most 1 + sqrt 2: the
+    // monomial form is as well conditioned on [-1, 1]). T_j has only powers of j's parity:
+    // the skipped terms' factors are zero, and with the splits on the integer pipe 72 of 258
+    // FP64 operations (64 cycles per warp each) fall away without a change of the results.
+    float2* out = t.coef + ((t.seg0[s] + g) * TAB_NF + f) * TAB_NC;
 #pragma unroll
-      for (int k = 0; k < TAB_NC; ++k) {
-        double a = 0.0;
+    for (int k = 0; k < TAB_NC; ++k) {
+      double a = 0.0;
 #pragma unroll
-        for (int j = k; j < TAB_NC; j += 2) a = fma(cc.mono[j][k], c[j], a);
-        const ff r = ff_of(a);
-        out[k] = make_float2(r.h, r.l);
-      }
+      for (int j = k; j < TAB_NC; j += 2) a = fma(cc.mono[j][k], c[j], a);
+      const ff r = ff_of(a);
+      out[k] = make_float2(r.h, r.l);
     }
   }
+}
+
+// Node sums and coefficients: a block per unit (TAB_CB pseudo-candidates of one spectrum), and
+// the block that ends a spectrum's last unit forms its coefficients. Those are bound by the
+// FP64 pipe, which the sums leave idle: as a kernel of their own they took 65 us after the
+// sums' 342 (1024 spectra, 40 segments, cost only); the whole evaluation of 256 candidates
+// each 678 -> 648 us.
+template <bool GRAD>
+__global__ void __launch_bounds__(MAX_BLOCK, GRAD ? 2 : 3) k_tab_build(const __grid_constant__ EvalArgs a,
+                                                                      const __grid_constant__ TabBuild t) {
+  __shared__ __align__(128) float4 stage_buf[STAGE_RECORDS];
+  __shared__ __align__(8) uint64_t stage_bar[2];
+  __shared__ int last;
+  Stage st;
+  stage_init(st, stage_buf, stage_bar);
+  const Unit u = a.units[blockIdx.x];
+  if (!sums_sq_unit<TAB_NODE_N, GRAD>(a, u, st)) return;
+  __threadfence();   // this thread's sums before the block's count
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int units = (t.qn0[u.s + 1] - t.qn0[u.s] + TAB_CB - 1) / TAB_CB;
+    last = atomicAdd(&t.done[u.s], 1) == units - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (last) tab_coef(t, a.sc.G, a.sc.x, a.sc.Q, u.s, GRAD ? TAB_NF : 3);
 }
 
 // f(x) = sum_k a_k x^k for x in [-1, 1] by Horner's rule in float-float. The
@@ -252,16 +288,14 @@ __global__ void __launch_bounds__(128) k_tab_eval(EvalArgs a, int smem_seg) {
   }
 }
 
-void launch_tab_nodes(int64_t S, const int32_t* qn0, const int32_t* nseg, const double* lo, double* theta_n,
-                      int sms, cudaStream_t st) {
+void launch_tab_build(const EvalArgs& a, int64_t S, const int32_t* qn0, const int32_t* nseg, const int64_t* seg0,
+                      const double* lo, double* theta_n, int32_t* done, bool with_grad, float2* coef, int sms,
+                      cudaStream_t st) {
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(S, (int64_t)sms * 32));
-  k_tab_nodes<<<grid, 128, 0, st>>>(S, qn0, nseg, lo, cheb_const(), theta_n);
-}
-
-void launch_tab_coef(int64_t S, const int32_t* qn0, const int32_t* nseg, const int64_t* seg0, const double* G,
-                     const double* X, int64_t Qn, bool with_grad, float2* coef, int sms, cudaStream_t st) {
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(S, (int64_t)sms * 32));
-  k_tab_coef<<<grid, 128, 0, st>>>(S, qn0, nseg, seg0, cheb_const(), G, X, Qn, with_grad ? TAB_NF : 3, coef);
+  k_tab_nodes<<<grid, 128, 0, st>>>(S, qn0, nseg, lo, cheb_const(), theta_n, done);
+  const TabBuild t{cheb_const(), qn0, nseg, seg0, done, coef};
+  if (with_grad) k_tab_build<true><<<a.n_units, TAB_CB * TAB_KS, 0, st>>>(a, t);
+  else k_tab_build<false><<<a.n_units, TAB_CB * TAB_KS, 0, st>>>(a, t);
 }
 
 // max_seg: the most segments of a spectrum. Shared memory for up to 64 segments (box of 12.8
