@@ -450,7 +450,7 @@ int debye_ctx::run_eval(EvalArgs a, const UnitGroups& g, bool mixed, int steps, 
   int rc;
   a.n_units = (int)g.units.size();
   if (a.n_units == 0) return DEBYE_OK;
-  if (a.ks < 1 || a.ks > 32 || (a.ks & (a.ks - 1)) || cb * a.ks > MAX_BLOCK)
+  if (!whole_warps(Layout{cb, a.ks}))
     return fail(DEBYE_EINTERNAL, "bad work layout (%d candidates x %d lanes)", cb, a.ks);
   const int gblock = warp_round(cb);
   auto grid_solve = [&](int n) { return std::max(1, std::min(n, sms * 32)); };
@@ -777,10 +777,7 @@ int debye_autotune(debye_handle h, const debye_spectra* sp, int32_t P, int32_t n
   if (sp->offsets_host && sp->S > 0) nsamp = sp->offsets_host[sp->S];
   snprintf(key, sizeof(key), "sms=%d prec=%d S=%lld P=%d nmax=%d samples=%lld", h->sms, h->opt.precision,
            (long long)sp->S, P, n_max, (long long)nsamp);
-  auto valid = [](Layout l, bool full) {
-    const bool pow2 = l.ks >= 1 && l.ks <= 32 && (l.ks & (l.ks - 1)) == 0;
-    return pow2 && l.cb >= 1 && l.cb * l.ks <= MAX_BLOCK && (!full || l.cb % 32 == 0);
-  };
+  auto valid = [](Layout l, bool full) { return whole_warps(l) && (!full || l.cb % 32 == 0); };
   auto report = [&]() {
     if (chosen) {
       chosen[0] = h->tuned.cb;
@@ -789,7 +786,7 @@ int debye_autotune(debye_handle h, const debye_spectra* sp, int32_t P, int32_t n
       chosen[3] = h->tuned_polish.ks;
     }
   };
-  if (cache_path) {  // "key | cb ks polish_cb polish_ks" lines
+  if (cache_path) {  // "key | cb ks polish_cb polish_ks" lines; one with a layout that no pass can run is passed over
     if (FILE* f = fopen(cache_path, "r")) {
       char line[256];
       while (fgets(line, sizeof(line), f)) {

@@ -19,6 +19,15 @@ struct Layout {
   int cb = 0, ks = 0;
 };
 
+// A layout that a pass can run: lanes a power of two up to 32, and a block of at most
+// MAX_BLOCK threads and of whole warps. The passes exchange values and vote over all 32
+// lanes of a warp, and the solves at their end deal candidates out to the block's warps: a
+// block of fewer than 32 threads would have none.
+__host__ __device__ constexpr bool whole_warps(Layout l) {
+  return l.ks >= 1 && l.ks <= 32 && (l.ks & (l.ks - 1)) == 0 && l.cb >= 1 && l.cb <= MAX_BLOCK &&
+         l.cb * l.ks <= MAX_BLOCK && l.cb * l.ks % 32 == 0;
+}
+
 // Work layout for spectra with `per_spectrum` candidates each, `total` in the
 // batch: `cb` candidates per unit and `ks` lanes per candidate. A population
 // that fills the GPU (about 2048 resident threads per SM) is a full population:
