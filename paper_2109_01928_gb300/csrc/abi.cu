@@ -147,6 +147,7 @@ int debye_ctx::load_plan(const debye_spectra* sp, Plan& pl, cudaStream_t st) {
   }
   if (pl.offs[0] != 0) return fail(DEBYE_EINVAL, "offsets[0] = %lld, expected 0", (long long)pl.offs[0]);
   pl.nmax_seen = 0;
+  pl.longest = 0;
   for (int64_t s = 0; s < pl.S; ++s) {
     if (pl.offs[s + 1] < pl.offs[s])
       return fail(DEBYE_EINVAL, "offsets not non-decreasing at spectrum %lld", (long long)s);
@@ -155,6 +156,7 @@ int debye_ctx::load_plan(const debye_spectra* sp, Plan& pl, cudaStream_t st) {
     if (pl.npol[s] < 1 || pl.npol[s] > NMAX)
       return fail(DEBYE_EINVAL, "n_poles[%lld] = %d outside 1..%d", (long long)s, pl.npol[s], NMAX);
     pl.nmax_seen = std::max(pl.nmax_seen, pl.npol[s]);
+    pl.longest = std::max(pl.longest, pl.offs[s + 1] - pl.offs[s]);
   }
   pl.n_samples = pl.offs[pl.S];
   return DEBYE_OK;
@@ -164,10 +166,10 @@ int debye_ctx::prep_spectra(const debye_spectra* sp, const Plan& pl, cudaStream_
   int rc;
   if ((rc = ensure(ws_kq, sizeof(float4) * (3 * pl.n_samples + granule_count(pl.n_samples, pl.S)), "sample planes"))) return rc;
   if ((rc = ensure(ws_h0, sizeof(double) * 2 * std::max<int64_t>(pl.S, 1), "h0"))) return rc;
-  launch_prep(pl.n_samples, pl.S, sp->offsets, sp->omega, sp->eps_re, sp->eps_im, sp->lo, sp->hi,
+  launch_prep(pl.n_samples, pl.S, pl.longest, sp->offsets, sp->omega, sp->eps_re, sp->eps_im, sp->lo, sp->hi,
               (float4*)ws_kq.p, (float4*)ws_kq.p + pl.n_samples, (float4*)ws_kq.p + 2 * pl.n_samples,
               (float4*)ws_kq.p + 3 * pl.n_samples, (double*)ws_h0.p, d_status, sms, st);
-  launches += pl.S > 0 ? (prep_merged(pl.n_samples, pl.S) ? 1 : 2) : 0;
+  launches += pl.S > 0 ? (prep_merged(pl.longest) ? 1 : 2) : 0;
   return check_launch("prep");
 }
 

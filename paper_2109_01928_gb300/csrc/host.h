@@ -20,6 +20,7 @@ struct Plan {
   int64_t S = 0;
   int64_t n_samples = 0;
   int32_t nmax_seen = 0;
+  int64_t longest = 0;   // the most samples of a spectrum
   std::vector<int64_t> offs;
   std::vector<int32_t> npol;
 };

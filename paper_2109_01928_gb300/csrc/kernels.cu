@@ -32,48 +32,92 @@ struct PrepSample {
   }
 };
 
-__global__ void k_prep_samples(int64_t n, const double* __restrict__ omega, const double* __restrict__ er,
-                               const double* __restrict__ ei, PrepPlanes planes, int* status) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    PrepSample(omega[k], er[k], ei[k], status).write(planes, k);
+// The bounds of a granule, a sample per lane: {smallest (omega 2^-30)^2, largest eps', largest
+// omega eps'', largest (omega 2^-30)^2}.
+struct PrepGranule {
+  float w2lo = INFINITY, w2hi = 0.f, e = 0.f, c = 0.f;   // neutral for the lanes past the spectrum's end
+  __device__ __forceinline__ void take(const PrepSample& smp) {
+    w2lo = w2hi = smp.w2.h;   // the factor of the bounds' test covers its rounding
+    e = smp.e.h;
+    c = smp.c.h;
+    if (!(e >= 0.f && e < INFINITY && c >= 0.f && c < INFINITY && w2lo >= 0.f)) e = c = INFINITY;
+  }
+  __device__ __forceinline__ void write(float4* at) {
+    for (int o = 16; o > 0; o >>= 1) {
+      w2lo = fminf(w2lo, __shfl_xor_sync(0xffffffffu, w2lo, o));
+      w2hi = fmaxf(w2hi, __shfl_xor_sync(0xffffffffu, w2hi, o));
+      e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
+      c = fmaxf(c, __shfl_xor_sync(0xffffffffu, c, o));
+    }
+    if ((threadIdx.x & 31) == 0) *at = make_float4(w2lo, e, c, w2hi);
+  }
+};
+static_assert(GRANULE == 32, "a granule is a warp's samples");
+
+// Planes and granules, PREP_RUN places of kg a warp's turn: the spectrum of the first is found
+// by bisection of the spectra's first places (they ascend), the others follow. Spread over
+// the whole grid whatever the spectra's lengths.
+constexpr int PREP_RUN = 4;
+__global__ void k_prep_samples(int64_t places, int64_t S, const int64_t* __restrict__ offsets,
+                               const double* __restrict__ omega, const double* __restrict__ er,
+                               const double* __restrict__ ei, float4* __restrict__ kg, PrepPlanes planes, int* status) {
+  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t warps = (int64_t)gridDim.x * blockDim.x >> 5;
+  for (int64_t g0 = warp * PREP_RUN; g0 < places; g0 += warps * PREP_RUN) {
+    int64_t s = 0, last = S - 1;
+    while (s < last) {
+      const int64_t m = (s + last + 1) >> 1;
+      if (granule_base(offsets[m], m) <= g0) s = m;
+      else last = m - 1;
+    }
+    for (int64_t g = g0; g < g0 + PREP_RUN && g < places; ++g) {
+      while (s + 1 < S && granule_base(offsets[s + 1], s + 1) <= g) ++s;
+      const int64_t a = offsets[s], b = offsets[s + 1], k0 = a + (g - granule_base(a, s)) * GRANULE;
+      if (k0 >= b) continue;   // a place that the spectrum does not fill
+      const int64_t k = k0 + (threadIdx.x & 31);
+      PrepGranule gr;
+      if (k < b) {
+        const PrepSample smp(omega[k], er[k], ei[k], status);
+        smp.write(planes, k);
+        gr.take(smp);
+      }
+      gr.write(kg + g);
+    }
+  }
 }
 
-// One block per spectrum; each warp's 32 samples of an iteration are one granule. PLANES:
-// the samples' planes are written here too, one launch and one read of the samples for both
-// (a long spectrum would be one block's work, so there k_prep_samples spreads the samples).
-template <bool PLANES>
+// h0 and b^T b, one block per spectrum. MERGED: the planes and granules too (each warp's 32
+// samples of an iteration are one granule), one launch and one read of the samples for both.
+// A long spectrum's would be one block's work: there k_prep_samples makes them.
+template <bool MERGED>
 __global__ void k_prep_spectra(int64_t S, const int64_t* __restrict__ offsets, const double* __restrict__ omega,
                                const double* __restrict__ er, const double* __restrict__ ei,
                                const double* __restrict__ lo, const double* __restrict__ hi,
                                double* __restrict__ h0, double* __restrict__ bb, float4* __restrict__ kg,
                                PrepPlanes planes, int* status) {
-  static_assert(GRANULE == 32, "a granule is a warp's samples");
   __shared__ double red[32], red2[32];
   for (int64_t s = blockIdx.x; s < S; s += gridDim.x) {
     const int64_t a = offsets[s], b = offsets[s + 1];
     double acc = 0.0, acc2 = 0.0;
-    for (int64_t k0 = a + (threadIdx.x & ~31u); k0 < b; k0 += blockDim.x) {
-      const int64_t k = k0 + (threadIdx.x & 31);
-      float w2lo = INFINITY, w2hi = 0.f, e = 0.f, c = 0.f;   // neutral for the lanes past the spectrum's end
-      if (k < b) {
-        const double w = omega[k], r = er[k], i = ei[k];
-        acc += r;
-        acc2 = fma(r, r, fma(i, i, acc2));
-        const PrepSample smp(w, r, i, status);
-        if (PLANES) smp.write(planes, k);
-        w2lo = w2hi = smp.w2.h;   // the factor of the bounds' test covers its rounding
-        e = smp.e.h;
-        c = smp.c.h;
-        if (!(e >= 0.f && e < INFINITY && c >= 0.f && c < INFINITY && w2lo >= 0.f)) e = c = INFINITY;
+    if constexpr (!MERGED) {
+      for (int64_t k = a + threadIdx.x; k < b; k += blockDim.x) {
+        acc += er[k];
+        acc2 = fma(er[k], er[k], fma(ei[k], ei[k], acc2));
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        w2lo = fminf(w2lo, __shfl_xor_sync(0xffffffffu, w2lo, o));
-        w2hi = fmaxf(w2hi, __shfl_xor_sync(0xffffffffu, w2hi, o));
-        e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
-        c = fmaxf(c, __shfl_xor_sync(0xffffffffu, c, o));
+    } else {
+      for (int64_t k0 = a + (threadIdx.x & ~31u); k0 < b; k0 += blockDim.x) {
+        const int64_t k = k0 + (threadIdx.x & 31);
+        PrepGranule gr;
+        if (k < b) {
+          const double r = er[k], i = ei[k];
+          acc += r;
+          acc2 = fma(r, r, fma(i, i, acc2));
+          const PrepSample smp(omega[k], r, i, status);
+          smp.write(planes, k);
+          gr.take(smp);
+        }
+        gr.write(kg + granule_base(a, s) + (k0 - a) / GRANULE);
       }
-      if ((threadIdx.x & 31) == 0) kg[granule_base(a, s) + (k0 - a) / GRANULE] = make_float4(w2lo, e, c, w2hi);
     }
     for (int o = 16; o > 0; o >>= 1) {
       acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -354,19 +398,20 @@ __global__ void __launch_bounds__(256) k_grad_finish(EvalArgs a, double* grad) {
 }
 
 // ------------------------------------------------------------------ host launchers
-void launch_prep(int64_t n_samples, int64_t S, const int64_t* offsets, const double* omega,
+void launch_prep(int64_t n_samples, int64_t S, int64_t longest, const int64_t* offsets, const double* omega,
                  const double* er, const double* ei, const double* lo, const double* hi,
                  float4* kq0, float4* kq1, float4* kq2, float4* kg, double* h0, int* status, int sms,
                  cudaStream_t st) {
   const PrepPlanes planes{kq0, kq1, kq2};
   if (S <= 0) return;
   const int grid = (int)std::min<int64_t>(S, (int64_t)sms * 8);
-  if (prep_merged(n_samples, S)) {
+  if (prep_merged(longest)) {
     k_prep_spectra<true><<<grid, 256, 0, st>>>(S, offsets, omega, er, ei, lo, hi, h0, h0 + S, kg, planes, status);
     return;
   }
-  const int sgrid = (int)std::min<int64_t>((n_samples + 255) / 256, (int64_t)sms * 16);
-  k_prep_samples<<<sgrid, 256, 0, st>>>(n_samples, omega, er, ei, planes, status);
+  const int64_t places = granule_count(n_samples, S), per_block = 8 * PREP_RUN;
+  const int sgrid = (int)std::min<int64_t>((places + per_block - 1) / per_block, (int64_t)sms * 16);
+  k_prep_samples<<<sgrid, 256, 0, st>>>(places, S, offsets, omega, er, ei, kg, planes, status);
   k_prep_spectra<false><<<grid, 256, 0, st>>>(S, offsets, omega, er, ei, lo, hi, h0, h0 + S, kg, planes, status);
 }
 

@@ -77,9 +77,13 @@ inline void launch_pass(int N, int phase, const EvalArgs& a, int grid, int block
 
 // kq0, kq1, kq2: [n_samples] each, the sample planes of EvalArgs; kg: [granule_count];
 // h0: [2 S] doubles, sum_k eps'_k per spectrum, then b^T b per spectrum.
-// One launch, or two (prep_merged false): spectra of more than 4096 samples on average.
-inline bool prep_merged(int64_t n_samples, int64_t S) { return n_samples <= 4096 * S; }
-void launch_prep(int64_t n_samples, int64_t S, const int64_t* offsets, const double* omega,
+// longest: the most samples of a spectrum. One launch, a block per spectrum, or two
+// (prep_merged false) where the longest spectrum would be too much work for one block:
+// whole evaluations of 2 candidates, one launch against two: 1000 samples each, 1 spectrum 54
+// and 58 us, 512 spectra 75 and 88; 4000 samples, 75 and 78, 125 and 133; 6000 samples, 1
+// spectrum 90 and 82, 64 spectra 94 and 86; 16000 samples, 148 and 126, 170 and 154.
+inline bool prep_merged(int64_t longest) { return longest <= 4096; }
+void launch_prep(int64_t n_samples, int64_t S, int64_t longest, const int64_t* offsets, const double* omega,
                  const double* er, const double* ei, const double* lo, const double* hi,
                  float4* kq0, float4* kq1, float4* kq2, float4* kg, double* h0, int* status, int sms,
                  cudaStream_t st);

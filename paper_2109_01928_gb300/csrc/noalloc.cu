@@ -214,6 +214,8 @@ extern "C" int debye_eval_population_noalloc(const debye_options* opt_in, const 
   }
   begin[N_BUCKETS] = n_units;
   const int64_t n_samples = offs[S];
+  int64_t longest = 0;
+  for (int64_t s = 0; s < S; ++s) longest = std::max(longest, offs[s + 1] - offs[s]);
 
   // carve the fixed scratch: status, units, per-sample, per-spectrum and per-candidate arrays
   void* base = nullptr;
@@ -265,7 +267,7 @@ extern "C" int debye_eval_population_noalloc(const debye_options* opt_in, const 
     cudaGetLastError();
     return fail_msg(DEBYE_ECUDA, err, err_len, cudaGetErrorString(e));
   }
-  launch_prep(n_samples, S, sp->offsets, sp->omega, sp->eps_re, sp->eps_im, sp->lo, sp->hi, kqa,
+  launch_prep(n_samples, S, longest, sp->offsets, sp->omega, sp->eps_re, sp->eps_im, sp->lo, sp->hi, kqa,
               kqa + n_samples, kqb, kg, h0, status, sms, st);
 
   EvalArgs a{};
