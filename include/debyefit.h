@@ -311,7 +311,8 @@ int debye_sync(debye_handle h, cudaStream_t stream);
  * launches. Per kind the library accumulates the number of passes, the summed
  * event time (ms) and the algorithmic FLOPs of the work, per candidate and
  * frequency sample (FMA counted as 2): mixed precision, 54N for the float-float
- * column-sum pass (103N with the derivative sums of a gradient evaluation);
+ * column-sum pass (103N with the derivative sums of a gradient evaluation), the count
+ * of its general form (runs of samples in order take fewer additions: 48N, 91N);
  * FP64, 4N + 2(N+2)^2 for the Gram pass (basis build plus the unique
  * Gram/right-hand-side products) and 13N + 5 for the residual pass.
  * Passes restricted by an activity mask (the polish line search and its accepted
