@@ -183,9 +183,8 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
   // generation 0: initial positions (the same for both methods), evaluation, bests
   launch_pso_init(sa, h->sms, st); ++h->launches;
   if ((rc = h->run_eval(ea, g, mixed, steps, cost, nullptr, nullptr, h->sb_eval.g1, cb, st))) return rc;
-  // the swarm: bests and the next generation's move in one kernel where a block takes a
-  // whole population
-  const bool swarm_step = !evolve && !anneal && P <= PSO_STEP_MAX_P;
+  // the swarm: bests and the next generation's move in one kernel, or in two
+  const bool swarm_step = !evolve && !anneal && pso_step_fused(pl.S, P, pl.nmax_seen);
   if (!swarm_step) {
     launch_pso_best(sa, cost, h->sms, st); ++h->launches;
     if (anneal) {

@@ -116,7 +116,7 @@ __device__ __forceinline__ double move_one(const MoveCoef& c, uint64_t key1, uin
 // and the keys' prefixes, the same for a whole spectrum, are formed once per block. What is
 // left is the FP64 pipe: 7 operations per coordinate (10 with coefficients that are no
 // powers of two), 64 cycles per warp each. 1024 spectra x 256 particles, N 2-12: 83 -> 57
-// us. It serves populations beyond PSO_STEP_MAX_P; smaller ones take k_pso_step.
+// us. It serves what pso_step_fused turns away.
 constexpr int MOVE_BLOCK = 256;
 __global__ void __launch_bounds__(MOVE_BLOCK) k_pso_move(SwarmArgs a, int chunks) {
   __shared__ uint64_t prefix[2];
@@ -396,10 +396,11 @@ __global__ void k_pso_best(SwarmArgs a, const double* __restrict__ cost) {
 // k_pso_best and the move of the next generation in one kernel, one block per spectrum: the
 // bests and the move read the same rows, and a generation of a small batch is bound by the
 // launches' latencies (one spectrum of 64 particles: 13.4 us for the two, with the counter's
-// kernel, against 6.8; 1024 spectra x 256: 73 against 50). The generation just
-// evaluated is gens[s], advanced by the spectrum's own block. Improved rows are copied to
-// the personal bests as the move passes over them; the global best's row is taken to shared
-// memory first, since its particle moves too.
+// kernel, against 6.8; 1024 spectra x 256: 73 against 50); where a spectrum has more work
+// than that, pso_step_fused. The generation just evaluated is gens[s], advanced by the
+// spectrum's own block. Improved rows are copied to the personal bests as the move passes
+// over them; the global best's row is taken to shared memory first, since its particle
+// moves too.
 constexpr int STEP_BLOCK = 256;
 template <bool MOVE>
 __global__ void __launch_bounds__(STEP_BLOCK) k_pso_step(SwarmArgs a, const double* __restrict__ cost) {

@@ -72,6 +72,18 @@ void launch_pso_best(const SwarmArgs& a, const double* cost, int sms, cudaStream
 // Bests of the generation just evaluated and (move) the positions of the next one, for
 // populations of at most PSO_STEP_MAX_P.
 constexpr int PSO_STEP_MAX_P = 1024;
+// Whether a batch's generations take it, or k_pso_best and k_pso_move: it has one block per
+// spectrum, so with few spectra a population of many coordinates (particles x poles) leaves
+// the GPU idle, where the move of its own spreads over it. Whole fits, separate kernels
+// against one, ms: 1 spectrum, 100 generations, 64 particles x 3 poles 2.08 and 1.87, 128 x
+// 10 3.85 and 3.85, 256 x 10 3.90 and 4.29, 1024 x 20 7.75 and 13.15; 64 spectra, 128 x 10
+// 12.37 and 12.18, 200 x 10 (60 generations) 8.02 and 8.01, 512 x 10 21.8 and 22.4; 152
+// spectra, 256 x 20 53.3 and 53.3, 1024 x 20 92.4 and 97.6; 1024 spectra, 256 x 12 (60)
+// 26.8 and 25.9, 1024 x 20 (60) 365 and 356.
+inline bool pso_step_fused(int64_t S, int P, int n_max) {
+  const int64_t coords = (int64_t)P * n_max;
+  return P <= PSO_STEP_MAX_P && (coords <= 1280 || coords <= 32 * S);
+}
 void launch_pso_step(const SwarmArgs& a, const double* cost, bool move, int sms, cudaStream_t st);
 void launch_gen_advance(int* gen, cudaStream_t st);
 void launch_add_scalar(double* dst, double v, cudaStream_t st);
