@@ -19,12 +19,9 @@ using namespace debyefit;
 namespace {
 
 // Line search of the polish: the full step is evaluated first (with its gradient);
-// a line that rejects it evaluates POLISH_R further step lengths per backtracking round.
-// Where so few lines are polished that all their step lengths together leave the GPU
-// unfilled (one warp per candidate's solve, see solve_sums_by_warp), one round evaluates
-// every step length: the rounds after the first, idle as a rule, cost their launches only
-// (one spectrum, 8 lines: 7 launches fewer per iteration). A round is at most 32 trials.
-constexpr int POLISH_R = 8;
+// a line that rejects it evaluates POLISH_R further step lengths per backtracking round, or
+// all of them in one (polish_one_round): the rounds after the first, idle as a rule, cost
+// their launches only.
 
 struct GraphGuard {
   cudaGraph_t g = nullptr;
@@ -238,8 +235,8 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
     pa.L = pl.S * (int64_t)T;
     pa.R = POLISH_R;
     // (the failure counter counts evaluated candidates, so it keeps the rounds)
-    if (h->opt.lbfgs_max_trials > 1 + POLISH_R && h->opt.lbfgs_max_trials <= 33 && !se->n_failed &&
-        solve_sums_by_warp(pa.L * (h->opt.lbfgs_max_trials - 1), 0, h->sms))
+    if (!se->n_failed &&
+        polish_one_round(pa.L, h->opt.lbfgs_max_trials - 1, pl.nmax_seen, h->opt.precision, h->sms))
       pa.R = h->opt.lbfgs_max_trials - 1;
     pa.nmax = nmax;
     pa.m = h->opt.lbfgs_m;
@@ -292,9 +289,9 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
       ab[s] = (int32_t)(s * T);
       ae[s] = (int32_t)((s + 1) * T);
     }
-    // trial steps: POLISH_R candidates per work unit (a line's step lengths of a round), so
-    // that a unit whose line has stopped searching exits at once and an active one has no
-    // idle candidates
+    // trial steps: POLISH_R candidates per work unit (a line's step lengths of a round, or of
+    // one round for all, where a unit may hold the ends of two lines), so that a unit whose
+    // lines have stopped searching exits at once and an active one has few idle candidates
     int cba, ksa;
     const int cbp = POLISH_R, ksp = MAX_BLOCK / POLISH_R;
     if (h->tuned_polish.cb > 0) {   // debye_autotune's choice for this shape

@@ -85,6 +85,23 @@ inline bool pso_step_fused(int64_t S, int P, int n_max) {
   return P <= PSO_STEP_MAX_P && (coords <= 1280 || coords <= 32 * S);
 }
 void launch_pso_step(const SwarmArgs& a, const double* cost, bool move, int sms, cudaStream_t st);
+// Step lengths of a polish line evaluated in a round, and whether one round takes all
+// `trials` of them (at most 32). Its launches are saved then (one spectrum, 8 lines: 7 per
+// iteration), but a line that rejects every step evaluates all of them at once, so the GPU
+// has to have room: at most 256 trials per SM over all lines, and fewer where one costs more
+// (poles, and FP64). Whole fits, rounds against one round, ms, 8 lines per spectrum and 19
+// step lengths (the default): mixed, 1 spectrum, 3 poles 3.62 and 3.08; 64, 8 poles 7.99 and
+// 6.43; 128, 20 poles of 4000 samples 38.7 and 38.2; 256, 4 poles 3.48 and 3.03, 12 poles of
+// 1000 samples 12.6 and 13.3, 20 21.4 and 24.0. Tables, 256, 12 poles 4.83 and 4.55, 20 poles
+// 7.76 and 8.06. FP64 column sums, 64, 20 poles of 400 samples 104 and 96; 128, 12 poles 68.0
+// and 68.6, 20 poles 135 and 140; 256, 4 poles 30.2 and 29.2, 8 poles 64.2 and 67.2.
+constexpr int POLISH_R = 8;
+inline bool polish_one_round(int64_t lines, int trials, int n_max, int precision, int sms) {
+  const int64_t all = lines * trials, room = precision == DEBYE_PREC_MIXED_TABLE ? 5120
+                                             : precision == DEBYE_PREC_MIXED     ? 3584
+                                                                                 : 2560;
+  return trials > POLISH_R && trials <= 32 && all <= 256 * (int64_t)sms && all * (n_max + 8) <= room * sms;
+}
 void launch_gen_advance(int* gen, cudaStream_t st);
 void launch_add_scalar(double* dst, double v, cudaStream_t st);
 void launch_topk(const SwarmArgs& a, const PolishArgs& pa, int sms, cudaStream_t st);

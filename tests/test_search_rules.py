@@ -40,6 +40,17 @@ def test_swarm_step_goes_by_coordinates_per_spectrum(rule):
     assert rule([f"pso_step_fused({s}ll, {p}, {n})" for s, p, n in cases]) == list(cases.values())
 
 
+def test_polish_round_goes_by_trials_and_poles(rule):
+    # (lines, trials, poles, precision) on 152 SMs
+    cases = {(8, 19, 3, "MIXED"): 1, (8, 8, 3, "MIXED"): 0, (8, 9, 3, "MIXED"): 1, (8, 32, 3, "MIXED"): 1,
+             (8, 33, 3, "MIXED"): 0, (8, 0, 3, "MIXED"): 0, (1024, 19, 20, "MIXED"): 1, (1025, 19, 20, "MIXED"): 0,
+             (2048, 19, 6, "MIXED"): 1, (2048, 19, 7, "MIXED"): 0, (2049, 19, 1, "MIXED"): 0,
+             (2048, 19, 12, "MIXED_TABLE"): 1, (2048, 19, 13, "MIXED_TABLE"): 0, (2049, 19, 1, "MIXED_TABLE"): 0,
+             (512, 19, 20, "FP64"): 1, (1024, 19, 12, "FP64"): 1, (1024, 19, 13, "FP64"): 0, (2048, 19, 2, "FP64"): 1,
+             (2048, 19, 3, "FP64_SUMS"): 0, (1 << 40, 32, 20, "FP64_SUMS"): 0}
+    assert rule([f"polish_one_round({l}ll, {t}, {n}, DEBYE_PREC_{p}, 152)" for l, t, n, p in cases]) == list(cases.values())
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("P,N", [(257, 5), (300, 7), (1024, 2)])
 def test_swarm_steps_of_both_forms_agree(P, N):
