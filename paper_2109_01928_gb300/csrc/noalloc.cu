@@ -254,7 +254,10 @@ extern "C" int debye_eval_population_noalloc(const debye_options* opt_in, const 
   // The granules (mixed precision) take plane 3's place; with hardly more samples than
   // spectra they do not fit there (n / 32 + S > n, so 16.6 B per spectrum at most) and take
   // the factor's (24 B per candidate at least), which only the FP64 path uses.
-  float4* kg = granule_count(n_samples, S) <= n_samples ? kqb + n_samples : (float4*)sc.L;
+  const bool granules_fit = granule_count(n_samples, S) <= n_samples;
+  if (!granules_fit && sizeof(float4) * granule_count(n_samples, S) > sizeof(double) * npk * Q)
+    return fail_msg(DEBYE_EINTERNAL, err, err_len, "no place for the granule records");
+  float4* kg = granules_fit ? kqb + n_samples : (float4*)sc.L;
 
   int sms = 1;
   int dev = 0;
