@@ -52,7 +52,7 @@ extern "C" {
 #define DEBYE_OK          0
 #define DEBYE_EINVAL     -1   /* bad argument (null pointer, size, bounds, N) */
 #define DEBYE_ECUDA      -2   /* a CUDA runtime call failed */
-#define DEBYE_ENOMEM     -3   /* device workspace allocation failed */
+#define DEBYE_ENOMEM     -3   /* allocation of device workspace or pinned host memory failed */
 #define DEBYE_ETIMEOUT   -4   /* a bounded device-side wait gave up */
 #define DEBYE_EINTERNAL  -5   /* inconsistent internal state */
 #define DEBYE_ENOTFINITE -6   /* non-finite frequency or target value on the device */
@@ -174,10 +174,16 @@ typedef struct {
 void debye_default_options(debye_options* opt);
 
 /* Create a handle on the current CUDA device. opt may be NULL (defaults).
+ * A handle holds 1 MiB of pinned host memory from its creation, four slots through
+ * which the plans of calls are uploaded. A larger plan (32 bytes per work unit, a
+ * block of candidates of one spectrum; in DEBYE_PREC_MIXED_TABLE also 16 bytes per
+ * spectrum) makes its slot grow, and the slot keeps that size until the handle is
+ * released. A call that evaluates on a stream that is being captured returns
+ * DEBYE_ECUDA.
  * Returns DEBYE_EINVAL for out-of-range options, DEBYE_ECUDA if no device. */
 int debye_fit_init(debye_handle* out, const debye_options* opt);
 
-/* Release a handle and its device workspaces. NULL is accepted. */
+/* Release a handle, its device workspaces and its pinned memory. NULL is accepted. */
 int debye_fit_destroy(debye_handle h);
 
 /* Target synthesis (Eqs. 3-7): write eps', eps'' of every spectrum from its model

@@ -32,7 +32,8 @@ struct UnitGroups {
 };
 
 // Pinned host memory that plans are written to and copied from: a slot's memory may be
-// written again once the copy out of it has run (ev).
+// written again once the copy out of it has run (ev). A slot that a larger plan needed keeps
+// that size until the handle is released.
 struct StageSlot {
   void* p = nullptr;
   size_t cap = 0;
