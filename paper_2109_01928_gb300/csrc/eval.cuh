@@ -484,15 +484,6 @@ struct PoleSums {
   }
 };
 
-// A same-sign sum h + l less its bias, one for each of the group's ks lanes. The FP32
-// difference h - ks is exact below 2^24, where 1 is a multiple of h's last bit; beyond (more
-// than 2^24 samples), infinite or NaN, the difference is formed in FP64, in a call, so that
-// the FP64 pipe is left alone elsewhere.
-__device__ __forceinline__ bool unbias_exact(float h) { return h < 0x1p24f; }
-static __device__ __noinline__ double unbias_plain(float h, float l, int ks) {
-  return ((double)h - (double)ks) + (double)l;
-}
-
 // S, h (and D, E) of one pole in FP64, stored in float-float with tau (or as they are:
 // sums_f64): tau at x[0], the sums at G[0], G[dn], G[2 dn], G[3 dn]. One copy of the code
 // per kernel, called for every pole.
@@ -503,21 +494,19 @@ static __device__ __noinline__ void sums_write(double* x, double* G, int64_t dn,
   const double tau = x[0];
   const double B = dbl_of(s.ch) + dbl_of(s.cl);
   const double h = (dbl_of(s.ah) + dbl_of(s.al)) + tau * B;
-  // S without its bias; its FP64 rounding is that of the low part
-  const bool exact = unbias_exact(s.sh);
+  // the bias is removed exactly (sh >= ks); the sum's FP64 rounding is that of its low part
   ff S;
   two_sum(__fsub_rn(s.sh, (float)ks), s.sl, S.h, S.l);
   double D = 0.0, E = 0.0;
   if constexpr (GRAD) {
-    const double U = unbias_exact(s.uh) ? dbl_of(__fsub_rn(s.uh, (float)ks)) + dbl_of(s.ul)
-                                        : unbias_plain(s.uh, s.ul, ks);
+    const double U = dbl_of(__fsub_rn(s.uh, (float)ks)) + dbl_of(s.ul);
     const double Vs = dbl_of(s.vh) + dbl_of(s.vl);
     const double W = dbl_of(s.wh) + dbl_of(s.wl);
     D = -2.0 * LN10 * U;
     E = LN10 * (-2.0 * Vs + tau * (B - 2.0 * W));
   }
   if (sums_f64) {
-    G[0] = exact ? dbl_of(S.h) + dbl_of(S.l) : unbias_plain(s.sh, s.sl, ks);
+    G[0] = dbl_of(S.h) + dbl_of(S.l);
     G[dn] = h;
     if constexpr (GRAD) {
       G[2 * dn] = D;
@@ -525,7 +514,7 @@ static __device__ __noinline__ void sums_write(double* x, double* G, int64_t dn,
     }
   } else {
     store_ff(x, 0, ff_of(tau));
-    store_ff(G, 0, exact ? ff_round53(S) : ff_of(unbias_plain(s.sh, s.sl, ks)));
+    store_ff(G, 0, ff_round53(S));
     store_ff(G, dn, ff_of(h));
     if constexpr (GRAD) {
       store_ff(G, 2 * dn, ff_of(D));
