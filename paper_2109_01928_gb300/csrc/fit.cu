@@ -236,7 +236,8 @@ int fit_impl(debye_handle h, const debye_spectra* sp, const debye_search* se, in
     pa.R = POLISH_R;
     // (the failure counter counts evaluated candidates, so it keeps the rounds)
     if (!se->n_failed &&
-        polish_one_round(pa.L, h->opt.lbfgs_max_trials - 1, pl.nmax_seen, h->opt.precision, h->sms))
+        polish_one_round(pa.L, h->opt.lbfgs_max_trials - 1, pl.nmax_seen, pl.longest, h->opt.precision,
+                         h->sms))
       pa.R = h->opt.lbfgs_max_trials - 1;
     pa.nmax = nmax;
     pa.m = h->opt.lbfgs_m;

@@ -81,26 +81,28 @@ constexpr int PSO_STEP_MAX_P = 1024;
 // spectra, 256 x 20 53.3 and 53.3, 1024 x 20 92.4 and 97.6; 1024 spectra, 256 x 12 (60)
 // 26.8 and 25.9, 1024 x 20 (60) 365 and 356.
 inline bool pso_step_fused(int64_t S, int P, int n_max) {
-  const int64_t coords = (int64_t)P * n_max;
-  return P <= PSO_STEP_MAX_P && (coords <= 1280 || coords <= 32 * S);
+  const int64_t coords = (int64_t)P * n_max;   // k_pso_move's blocks take 16 particles, 256 coordinates at a time
+  return P <= PSO_STEP_MAX_P && (coords <= (n_max > 16 ? 1536 : 1280) || coords <= 32 * S);
 }
 void launch_pso_step(const SwarmArgs& a, const double* cost, bool move, int sms, cudaStream_t st);
 // Step lengths of a polish line evaluated in a round, and whether one round takes all
 // `trials` of them (at most 32). Its launches are saved then (one spectrum, 8 lines: 7 per
 // iteration), but a line that rejects every step evaluates all of them at once, so the GPU
 // has to have room: at most 256 trials per SM over all lines, and fewer where one costs more
-// (poles, and FP64). Whole fits, rounds against one round, ms, 8 lines per spectrum and 19
-// step lengths (the default): mixed, 1 spectrum, 3 poles 3.62 and 3.08; 64, 8 poles 7.99 and
-// 6.43; 128, 20 poles of 4000 samples 38.7 and 38.2; 256, 4 poles 3.48 and 3.03, 12 poles of
-// 1000 samples 12.6 and 13.3, 20 21.4 and 24.0. Tables, 256, 12 poles 4.83 and 4.55, 20 poles
-// 7.76 and 8.06. FP64 column sums, 64, 20 poles of 400 samples 104 and 96; 128, 12 poles 68.0
-// and 68.6, 20 poles 135 and 140; 256, 4 poles 30.2 and 29.2, 8 poles 64.2 and 67.2.
+// (poles; FP64; without tables, samples). Whole fits, rounds against one round, ms, 8 lines
+// per spectrum, 19 step lengths (the default): mixed, 1 spectrum, 3 poles 3.62 and 3.08; 64,
+// 8 poles 7.99 and 6.43; 128, 20 poles of 4000 samples 38.7 and 38.2; 192, 8 poles of 1000
+// 7.83 and 7.43, of 4000 17.4 and 17.8; 256, 4 poles 3.48 and 3.03, 8 poles of 1000 8.66 and
+// 8.70, 12 12.6 and 13.3, 20 21.4 and 24.0. Tables, 256, 12 poles 4.83 and 4.55, 20 poles 7.76
+// and 8.06. FP64 column sums, 64, 20 poles of 400 samples 104 and 96; 128, 12 poles 68.0 and
+// 68.6, 20 poles 135 and 140; 256, 4 poles 30.2 and 29.2, 8 poles 64.2 and 67.2.
 constexpr int POLISH_R = 8;
-inline bool polish_one_round(int64_t lines, int trials, int n_max, int precision, int sms) {
-  const int64_t all = lines * trials, room = precision == DEBYE_PREC_MIXED_TABLE ? 5120
-                                             : precision == DEBYE_PREC_MIXED     ? 3584
-                                                                                 : 2560;
-  return trials > POLISH_R && trials <= 32 && all <= 256 * (int64_t)sms && all * (n_max + 8) <= room * sms;
+inline bool polish_one_round(int64_t lines, int trials, int n_max, int64_t longest, int precision, int sms) {
+  if (trials <= POLISH_R || trials > 32 || lines * trials > 256 * (int64_t)sms) return false;
+  const double per_sm = (double)(lines * trials) / sms, work = per_sm * (n_max + 8);
+  if (precision == DEBYE_PREC_MIXED_TABLE) return work <= 5750.0;
+  if (precision == DEBYE_PREC_MIXED) return work <= 3000.0 || work * (double)(longest + 4000) <= 20.5e6;
+  return per_sm * (n_max + 2) <= 1800.0;
 }
 void launch_gen_advance(int* gen, cudaStream_t st);
 void launch_add_scalar(double* dst, double v, cudaStream_t st);

@@ -34,21 +34,24 @@ def rule(tmp_path_factory):
 
 
 def test_swarm_step_goes_by_coordinates_per_spectrum(rule):
-    cases = {(1, 64, 3): 1, (1, 64, 20): 1, (1, 128, 10): 1, (1, 129, 10): 0, (1, 1024, 1): 1, (1, 1024, 20): 0,
+    cases = {(1, 64, 3): 1, (1, 64, 20): 1, (1, 128, 10): 1, (1, 129, 10): 0, (1, 80, 16): 1, (1, 81, 16): 0, (5, 77, 18): 1, (1, 77, 20): 0, (1, 1024, 1): 1, (1, 1024, 20): 0,
              (40, 128, 10): 1, (41, 131, 10): 1, (64, 200, 10): 1, (64, 205, 10): 0, (152, 243, 20): 1,
              (152, 244, 20): 0, (1024, 256, 12): 1, (1024, 1024, 20): 1, (1024, 1025, 1): 0, (1 << 20, 1025, 20): 0}
     assert rule([f"pso_step_fused({s}ll, {p}, {n})" for s, p, n in cases]) == list(cases.values())
 
 
 def test_polish_round_goes_by_trials_and_poles(rule):
-    # (lines, trials, poles, precision) on 152 SMs
-    cases = {(8, 19, 3, "MIXED"): 1, (8, 8, 3, "MIXED"): 0, (8, 9, 3, "MIXED"): 1, (8, 32, 3, "MIXED"): 1,
-             (8, 33, 3, "MIXED"): 0, (8, 0, 3, "MIXED"): 0, (1024, 19, 20, "MIXED"): 1, (1025, 19, 20, "MIXED"): 0,
-             (2048, 19, 6, "MIXED"): 1, (2048, 19, 7, "MIXED"): 0, (2049, 19, 1, "MIXED"): 0,
-             (2048, 19, 12, "MIXED_TABLE"): 1, (2048, 19, 13, "MIXED_TABLE"): 0, (2049, 19, 1, "MIXED_TABLE"): 0,
-             (512, 19, 20, "FP64"): 1, (1024, 19, 12, "FP64"): 1, (1024, 19, 13, "FP64"): 0, (2048, 19, 2, "FP64"): 1,
-             (2048, 19, 3, "FP64_SUMS"): 0, (1 << 40, 32, 20, "FP64_SUMS"): 0}
-    assert rule([f"polish_one_round({l}ll, {t}, {n}, DEBYE_PREC_{p}, 152)" for l, t, n, p in cases]) == list(cases.values())
+    # (lines, trials, poles, longest spectrum, precision) on 152 SMs
+    cases = {(8, 19, 3, 50, "MIXED"): 1, (8, 8, 3, 50, "MIXED"): 0, (8, 9, 3, 50, "MIXED"): 1, (8, 32, 3, 50, "MIXED"): 1,
+             (8, 33, 3, 50, "MIXED"): 0, (8, 0, 3, 50, "MIXED"): 0, (8, 19, 20, 1 << 20, "MIXED"): 1,
+             (512, 19, 20, 1 << 30, "MIXED"): 1, (1024, 19, 20, 4000, "MIXED"): 0, (1024, 19, 20, 1000, "MIXED"): 1, (2048, 19, 8, 1000, "MIXED"): 1, (2048, 19, 8, 1200, "MIXED"): 0,
+             (1496, 19, 16, 180, "MIXED"): 1, (2048, 19, 12, 1000, "MIXED"): 0, (2049, 19, 1, 2, "MIXED"): 0,
+             (2048, 19, 14, 4000, "MIXED_TABLE"): 1, (2048, 19, 15, 50, "MIXED_TABLE"): 0,
+             (2049, 19, 1, 50, "MIXED_TABLE"): 0, (512, 19, 20, 4000, "FP64"): 1, (1024, 19, 12, 400, "FP64"): 1,
+             (1024, 19, 13, 400, "FP64"): 0, (2048, 19, 5, 50, "FP64"): 1, (2048, 19, 6, 50, "FP64_SUMS"): 0,
+             (1 << 40, 32, 20, 1 << 30, "FP64_SUMS"): 0}
+    assert rule([f"polish_one_round({l}ll, {t}, {n}, {k}ll, DEBYE_PREC_{p}, 152)"
+                 for l, t, n, k, p in cases]) == list(cases.values())
 
 
 @pytest.mark.gpu
