@@ -494,7 +494,11 @@ static __device__ __noinline__ void sums_write(double* x, double* G, int64_t dn,
   const double tau = x[0];
   const double B = dbl_of(s.ch) + dbl_of(s.cl);
   const double h = (dbl_of(s.ah) + dbl_of(s.al)) + tau * B;
-  // the bias is removed exactly (sh >= ks); the sum's FP64 rounding is that of its low part
+  // The bias is removed exactly. A lane's sh, grown by terms of at most 1, stays at most 2^24
+  // (2^24 + 1 is a tie that rounds to 2^24; what is lost goes to sl), so the ks lanes' total is
+  // at most ks 2^24: its last bit is at most ks, a power of two, and sh - ks a multiple of it
+  // that needs no more bits than sh. The same holds for uh. The sum's FP64 rounding is then that
+  // of its low part.
   ff S;
   two_sum(__fsub_rn(s.sh, (float)ks), s.sl, S.h, S.l);
   double D = 0.0, E = 0.0;
