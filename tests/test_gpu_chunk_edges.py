@@ -18,7 +18,7 @@ NS = [1, 2, 3, 6, 7, 8, 12, 13, 20]
 @pytest.mark.parametrize("cb,lanes", [(64, 1), (32, 4), (16, 8), (4, 32)])
 def test_column_sums_at_chunk_ends(cb, lanes):
     from paper_2109_01928_gb300 import debyefit as D
-    P = 21
+    P = 33   # a warp and more: fewer do not take a forced layout
     b = W.mixed_batch(S=len(KS), seed=19, P=P, K_range=(max(KS), max(KS)), N_range=(2, 12))
     keep = np.concatenate([np.arange(b.offsets[s], b.offsets[s] + k) for s, k in enumerate(KS)])
     re, im = models.synthesize(b)
@@ -39,7 +39,7 @@ def test_column_sums_at_chunk_ends(cb, lanes):
         ref, _ = dls.cost_population(om, re[a:c], im[a:c], th[s, :, :N])
         assert np.max(np.abs(cost[s] - ref) / ref) <= 1e-5, (s, KS[s], N)
         assert np.max(np.abs(gcost[s] - ref) / ref) <= 1e-5, (s, KS[s], N)
-        for p in range(0, P, 10):
+        for p in range(0, P, 16):
             x = dls.damped_solve(dls.basis(om, th[s, p, :N]), dls.target(re[a:c], im[a:c]), dls.LAM_SEARCH)
             if np.min(np.abs(x[1:])) < 1e-6 * np.abs(x).max():
                 continue
